@@ -19,6 +19,7 @@
 #include "mg_bodies64.cuh"
 #include "mg_internal.h"
 #include "mg_solver.h"
+#include "mg_tile64.cuh"
 
 namespace mg {
 
@@ -68,6 +69,18 @@ __global__ void __launch_bounds__(256) kb_smooth64(const BItem* __restrict__ ite
                                                    int colour) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
+  __shared__ TileShared S;
+  if (it.n >= kTileMinSide) {
+    const dim3 g = tile_grid(it.n);
+    const unsigned b = (unsigned)blk, r = b / g.x;
+    const int x0 = (int)(b - r * g.x) * kTileX, y0 = (int)(r % g.y) * kTileY,
+              z0 = (int)(r / g.y) * kTileZ;
+    if (it.f)
+      b_smooth_tile64<true>(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, x0, y0, z0, S);
+    else
+      b_smooth_tile64<false>(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, x0, y0, z0, S);
+    return;
+  }
   b_smooth_colour64(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, blk);
 }
 
@@ -183,12 +196,18 @@ __global__ void __launch_bounds__(256) kb_coarsest_corr32(const BItem* __restric
 // Host side
 // ---------------------------------------------------------------------------
 // T_HAND: the outer residual hand-off, kHandoffCells cells per thread
-enum ListType { T_SMOOTH = 0, T_RR, T_CELL, T_CCELL, T_ONE, T_HAND, T_NTYPES };
+// T_SM64: the FP64 colour stages, in tiles from kTileMinSide on
+enum ListType { T_SMOOTH = 0, T_RR, T_CELL, T_CCELL, T_ONE, T_HAND, T_SM64, T_NTYPES };
 
 static long long blocks_of(ListType t, int n) {
   const long long cells = (long long)n * n * n;
   switch (t) {
     case T_SMOOTH: return (cells / 4 + 255) / 256;
+    case T_SM64: {
+      if (n < kTileMinSide) return (cells / 4 + 255) / 256;
+      const dim3 g = tile_grid(n);
+      return (long long)g.x * g.y * g.z;
+    }
     case T_RR: return (cells / 8 + 255) / 256;
     case T_CELL: return (cells + 255) / 256;
     case T_CCELL: return (cells / 8 + 255) / 256;
@@ -392,7 +411,7 @@ struct BatchCycle {
   // ---- FP64 ----
   void smooth64(int l, int sweeps) const {
     for (int s = 0; s < sweeps; ++s)
-      for (int c = 0; c < 4; ++c) launch(L(l, T_SMOOTH, P_DESC), 256, kb_smooth64, c);
+      for (int c = 0; c < 4; ++c) launch(L(l, T_SM64, P_DESC), 256, kb_smooth64, c);
   }
   void part_a64() const {
     smooth64(0, o->nu_pre);

@@ -18,15 +18,56 @@ __device__ __forceinline__ double smooth_scalar64(const LevelScalars* __restrict
                            : -c.h2_6 * (c.mode == OP_SQRT ? sc->lambda - c.k2 : sc->lambda);
 }
 
+// phi += omega (v - phi), the relaxed step (omega < 1).
+static __device__ __noinline__ void relax64(double* phi, double v, double omega) {
+  const double old = *phi;
+  *phi = fma(omega, v - old, old);
+}
+
+// The update of cell (i,j,k) of a colour stage:
+//   phi_new = (Sx + Sy + Sz - h^2 (D + f + lambda)) / 6.
+// In the sqrt form, D = k2s sqrt(q) - k2, so phi_new = upd_s sqrt(q) + (Sx+Sy+Sz)/6 -
+// h^2 f/6 + C with the block-wide C = -h^2 (lambda - k2)/6 (s_c).
+__device__ __forceinline__ void cell_smooth64_at(int n, double* __restrict__ phi,
+                                                 const double* __restrict__ src,
+                                                 const double* __restrict__ f, double s_c,
+                                                 const OpConst64& c, int i, int j, int k) {
+  const long long id = lidx(i, j, k, n);
+  auto nbr = [&] { return nbr_offsets(i, j, k, n); };
+  if (c.mode == OP_GENW) {
+    const double old = phi[id];
+    const double v = genw_newton(gather_at(phi + id, nbr()), old, src[id],
+                                 (f ? f[id] : 0.0) + s_c, c);
+    phi[id] = not_one(c.omega) ? fma(c.omega, v - old, old) : v;
+    return;
+  }
+  long long b[18];
+  gather_bits(phi + id, nbr(), b);
+  const double sv = src[id];
+  const double fv = f ? f[id] : 0.0;
+  double face, M;
+  stencil_forms(phi + id, nbr, b, c.mode != OP_LINEAR, face, M);
+  double acc = fma(fv, -c.h2_6, s_c);
+  if (c.mode == OP_SQRT) {
+    acc = fma(c.upd_s, sqrt_clamped_fix(fma(c.e1, M, sv)), acc);
+  } else {
+    double q;
+    bool g;
+    acc = fma(-c.h2_6, root_of_M(M, sv, c, q, g), acc);
+  }
+  const double v = fma(face, 1.0 / 6.0, acc);
+  if (not_one(c.omega))
+    relax64(phi + id, v, c.omega);
+  else
+    phi[id] = v;
+}
+
 // One cell of a colour stage: t indexes the colour's n^3/4 cells; t >= n^3/4 does
 // nothing.
 __device__ __forceinline__ void cell_smooth64(int n, double* __restrict__ phi,
                                               const double* __restrict__ src,
                                               const double* __restrict__ f, double s_c,
                                               const OpConst64& c, int colour, long long t) {
-  // phi_new = (Sx + Sy + Sz - h^2 (D + f + lambda)) / 6.  In the sqrt form,
-  // D = k2s sqrt(q) - k2, so phi_new = upd_s sqrt(q) + (Sx+Sy+Sz)/6 - h^2 f/6 + C with
-  // the block-wide C = -h^2 (lambda - k2)/6 (s_c).
   const int hn = n >> 1;
   const long long total = (long long)hn * hn * n;
   if (t >= total) return;
@@ -34,31 +75,7 @@ __device__ __forceinline__ void cell_smooth64(int n, double* __restrict__ phi,
   split3((unsigned)t, hn, m, jj, k);
   const int i = 2 * m + ((colour ^ k) & 1);
   const int j = 2 * jj + (((colour >> 1) ^ k) & 1);
-  const long long id = lidx(i, j, k, n);
-  const StencilT<double> s = gather_periodic(phi, i, j, k, n);
-  if (c.mode == OP_GENW) {
-    const double old = phi[id];
-    const double v = genw_newton(s, old, src[id], (f ? f[id] : 0.0) + s_c, c);
-    phi[id] = not_one(c.omega) ? fma(c.omega, v - old, old) : v;
-    return;
-  }
-  const double lapnb = s.sx + s.sy + s.sz;
-  double acc = fma(lapnb, 1.0 / 6.0, s_c);
-  if (f) acc = fma(f[id], -c.h2_6, acc);
-  double v;
-  if (c.mode == OP_SQRT) {
-    const double B = fma(s.cxy, s.cxy, fma(s.cxz, s.cxz, s.cyz * s.cyz));
-    const double q = fma(c.e1h, half_A(s), fma(c.e2, B, src[id]));
-    v = fma(c.upd_s, sqrt_clamped(q), acc);
-  } else {
-    bool g;
-    v = fma(-c.h2_6, root_D(s, src[id], c, g), acc);
-  }
-  if (not_one(c.omega)) {
-    const double old = phi[id];
-    v = fma(c.omega, v - old, old);
-  }
-  phi[id] = v;
+  cell_smooth64_at(n, phi, src, f, s_c, c, i, j, k);
 }
 
 __device__ __forceinline__ void b_smooth_colour64(int n, double* __restrict__ phi,

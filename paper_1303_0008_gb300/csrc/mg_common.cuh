@@ -20,6 +20,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "mg_fix64.cuh"
+
 namespace mg {
 
 // How the root D is evaluated.
@@ -228,6 +230,90 @@ __device__ __forceinline__ double root_D(const StencilT<double>& s, double src,
   }
   const double u = fma(c.c1h, A2, fma(c.c2, B, src));
   const double q = fma(c.c3, u, 1.0);
+  guard = q < 0.0;
+  if (guard) return -c.k2;
+  return (2.0 * u) / (1.0 + sqrt(q));
+}
+
+// The 18 neighbours of a cell (and the cell itself with NV = 19) as bit patterns, in
+// the order x, y, z face pairs, the xy, xz, yz cells as (++, --, +-, -+), the centre.
+template <int NV>
+__device__ __forceinline__ void gather_bits(const double* __restrict__ c, const NbrOff& o,
+                                            long long (&b)[NV]) {
+  const int off[19] = {o.xp,        o.xm,        o.yp,        o.ym,        o.zp,
+                       o.zm,        o.xp + o.yp, o.xm + o.ym, o.xp + o.ym, o.xm + o.yp,
+                       o.xp + o.zp, o.xm + o.zm, o.xp + o.zm, o.xm + o.zp, o.yp + o.zp,
+                       o.ym + o.zm, o.yp + o.zm, o.ym + o.zp, 0};
+#pragma unroll
+  for (int k = 0; k < NV; ++k) b[k] = __double_as_longlong(c[off[k]]);
+}
+
+// stencil_forms of the cell at c in FP64, for values that fix_align refuses.  Not
+// inlined, as the other rare paths here: kept out of the way of the code that runs.
+static __device__ __noinline__ void stencil_forms_fp64(const double* c, NbrOff o, int nv,
+                                                       double* face, double* M) {
+  const StencilT<double> s = gather_at(c, o);
+  const double sum = s.sx + s.sy + s.sz;
+  const double B = fma(s.cxy, s.cxy, fma(s.cxz, s.cxz, s.cyz * s.cyz));
+  *face = nv == 19 ? sum - 6.0 * *c : sum;
+  *M = fma(0.375, B, 2.0 * half_A(s));
+}
+
+// What the operator needs of the stencil at `at` (b: its gather_bits, used up; nbr()
+// its offsets):
+//   face = Sx + Sy + Sz, with the centre (NV = 19) Sx + Sy + Sz - 6 phi;
+//   M = A + (3/8) B of Sigma_d h^4 = A/3 + B/8 (0 unless quad).
+template <int NV, typename Nbr>
+__device__ __forceinline__ void stencil_forms(const double* at, Nbr nbr, long long (&b)[NV],
+                                              bool quad, double& face, double& M) {
+  FixRef r;
+  M = 0.0;
+  if (!fix_align(b, r)) {
+    double fs, ms;
+    stencil_forms_fp64(at, nbr(), NV, &fs, &ms);
+    face = fs;
+    if (quad) M = ms;
+    return;
+  }
+  unsigned long long u[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) u[k] = (unsigned long long)b[k];
+  const unsigned long long sx = u[0] + u[1], sy = u[2] + u[3], sz = u[4] + u[5];
+  const unsigned long long sub = NV == 19 ? 6 * u[NV - 1] : (unsigned long long)r.off6;
+  face = fix_signed((long long)(sx + sy + sz - sub), r);
+  if (!quad) return;
+  const long long a[3] = {(long long)(sx - sy), (long long)(sx - sz), (long long)(sy - sz)};
+  const long long c[3] = {(long long)((u[6] + u[7]) - (u[8] + u[9])),
+                          (long long)((u[10] + u[11]) - (u[12] + u[13])),
+                          (long long)((u[14] + u[15]) - (u[16] + u[17]))};
+  int sh;
+  unsigned top;
+  const unsigned long long N = fix_quad(a, c, sh, top);
+  M = fix_double(N, 64 - 2 * sh + 2 * r.ue);
+}
+
+// sqrt_clamped with the square root of a normal q on the integer pipe.
+static __device__ __noinline__ double sqrt_clamped_rare(double q) { return sqrt_clamped(q); }
+
+__device__ __forceinline__ double sqrt_clamped_fix(double q) {
+  const unsigned e = (unsigned)(__double_as_longlong(q) >> 52);  // sign and exponent
+  return e - 1u < 2046u ? sqrt_fix_normal(q) : sqrt_clamped_rare(q);
+}
+
+// The root D of Eq. two_branch from M (stencil_forms) and the source term; q is the
+// discriminant (1 in the linear mode) and guard whether it is negative.
+__device__ __forceinline__ double root_of_M(double M, double src, const OpConst64& c, double& q,
+                                            bool& guard) {
+  q = 1.0;
+  guard = false;
+  if (c.mode == OP_LINEAR) return src;
+  if (c.mode == OP_SQRT) {
+    q = fma(c.e1, M, src);
+    guard = neg_guard(q);
+    return fma(c.k2s, sqrt_clamped_fix(q), -c.k2);
+  }
+  const double u = fma(c.c1, M, src);
+  q = fma(c.c3, u, 1.0);
   guard = q < 0.0;
   if (guard) return -c.k2;
   return (2.0 * u) / (1.0 + sqrt(q));

@@ -1,0 +1,276 @@
+// The operator's double-precision arithmetic on the integer and FP32 pipes.
+//
+// GB300 retires 2 FP64 lane-operations per SM and clock, so one FP64 warp instruction
+// holds its scheduler's FP64 unit for 64 cycles; an integer one takes 1 to 2.  A cell of
+// the operator needs 18 neighbours, 14 additions, six squares and a square root, about 33
+// FP64 instructions.  Here everything but three fused multiply-adds runs in 64-bit
+// integers, with no step less exact than its FP64 form:
+//   fix_align   the neighbours as integers of one unit.  Values of one sign and binade
+//               (the usual case: the field varies by a few percent over a stencil) need
+//               no conversion at all: their bit patterns differ by exactly the
+//               differences of their significands.  Values of one sign and near
+//               binades are shifted up, exactly; others are shifted to the largest
+//               exponent, with 7 more bits below.
+//   sums        exact (FP64 rounds each to half a unit in the last place of the field).
+//   fix_quad    the quadratic form of Sigma_d as a 62-bit integer, error below 2^-53.
+//   sqrt_fix    square root to about 2^-61 from the FP32 reciprocal square root and two
+//               exact integer residuals.
+//   fix_double  back to FP64, rounded once.
+// Cells whose values have no such form (all zero, infinities, NaN, exponents whose
+// squares leave the FP64 range) keep the FP64 code.  Every function depends on its arguments alone, so
+// all kernels that update a cell give the same bits.
+#pragma once
+
+#include <cstdint>
+#include <cstring>
+
+#ifdef __CUDACC__
+#include <cuda_runtime.h>
+#define MG_HD __host__ __device__ __forceinline__
+#else
+#define MG_HD inline
+#endif
+
+namespace mg {
+
+MG_HD long long fix_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return __double_as_longlong(x);
+#else
+  long long b;
+  std::memcpy(&b, &x, 8);
+  return b;
+#endif
+}
+
+MG_HD double fix_from_bits(long long b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double(b);
+#else
+  double x;
+  std::memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+
+MG_HD int fix_hi(long long b) { return (int)(b >> 32); }
+
+MG_HD int fix_clz32(unsigned x) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)x);
+#else
+  return x ? __builtin_clz(x) : 32;
+#endif
+}
+
+MG_HD int fix_clz64(unsigned long long x) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)x);
+#else
+  return x ? __builtin_clzll(x) : 64;
+#endif
+}
+
+MG_HD float fix_float(unsigned b) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float x;
+  std::memcpy(&x, &b, 4);
+  return x;
+#endif
+}
+
+// Shifts by 0 ... 31 of the 64-bit value hi:lo, word by word: the 64-bit operators cost
+// two to three times as many instructions where the amount is not known.
+MG_HD unsigned fix_shl_hi(unsigned lo, unsigned hi, int s) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_l(lo, hi, s);
+#else
+  return (unsigned)((((unsigned long long)hi << 32 | lo) << s) >> 32);
+#endif
+}
+MG_HD unsigned fix_shr_lo(unsigned lo, unsigned hi, int s) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_r(lo, hi, s);
+#else
+  return (unsigned)(((unsigned long long)hi << 32 | lo) >> s);
+#endif
+}
+MG_HD unsigned long long fix_words(unsigned lo, unsigned hi) {
+  return (unsigned long long)hi << 32 | lo;
+}
+
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ float fix_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ int fix_rint(float x) { return __float2int_rn(x); }
+#else
+float fix_rsqrt(float x);  // host checks provide one with the error of the device's
+inline int fix_rint(float x) {
+  return x >= 2147483648.f ? 2147483647 : (int)__builtin_llrint((double)x);
+}
+#endif
+
+// How the integers of a stencil read: value = (-1)^neg (integer - offset) 2^ue, where the
+// offset cancels in every difference; off6 is six times it.
+struct FixRef {
+  long long off6;
+  int ue;
+  bool neg;
+};
+
+// Exponent fields whose squares, scaled by any shift of fix_quad, stay normal doubles.
+constexpr int kFixMinExp = 640, kFixMaxExp = 1470;
+
+// Replace the bit patterns b[] by integers of one unit; false when the values have no
+// such form (b is then unchanged).
+template <int NV>
+MG_HD bool fix_align(long long (&b)[NV], FixRef& r) {
+  const int h0 = fix_hi(b[0]);
+  int diff = 0;
+#pragma unroll
+  for (int k = 1; k < NV; ++k) diff |= fix_hi(b[k]) ^ h0;
+  const unsigned se = (unsigned)h0 >> 20;  // sign and exponent
+  const int e0 = (int)(se & 0x7ffu);
+  if ((diff & (int)0xfff00000) == 0 && e0 >= kFixMinExp && e0 <= kFixMaxExp) {
+    r.off6 = (long long)((unsigned long long)(6u * (se - 1u)) << 52);
+    r.ue = e0 - 1075;
+    r.neg = h0 < 0;
+    return true;
+  }
+  if (diff >= 0 && e0 >= kFixMinExp + 3 && e0 <= kFixMaxExp - 7) {
+    // one sign: significands shifted up from three binades below the first value's
+    const unsigned lo = se - 3u;
+    unsigned d[NV], far = 0;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      d[k] = ((unsigned)fix_hi(b[k]) >> 20) - lo;
+      far |= d[k];
+    }
+    if (far <= 7u) {
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+        b[k] = (long long)((((unsigned long long)b[k] & 0xfffffffffffffULL) | 0x10000000000000ULL)
+                           << d[k]);
+      r.off6 = 0;
+      r.ue = e0 - 1078;
+      r.neg = h0 < 0;
+      return true;
+    }
+  }
+  int em = 0;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const int e = fix_hi(b[k]) & 0x7ff00000;
+    em = e > em ? e : em;
+  }
+  if (em < (kFixMinExp << 20) || em > (kFixMaxExp << 20)) return false;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const int h = fix_hi(b[k]);
+    int d = (em - (h & 0x7ff00000)) >> 20;
+    d = d > 63 ? 63 : d;
+    const long long s = b[k] >> 63;
+    const unsigned long long m =
+        (((unsigned long long)b[k] & 0xfffffffffffffULL) | 0x10000000000000ULL) << 7;
+    b[k] = (long long)((m >> d) ^ (unsigned long long)s) - s;
+  }
+  r.off6 = 0;
+  r.ue = (em >> 20) - 1082;
+  r.neg = false;
+  return true;
+}
+
+// (hi:lo + 2^9) 2^-10, the significand of a double with its leading bit at 2^62 rounded,
+// under the exponent field be (less one: the leading bit adds it) and the sign bit.
+MG_HD double fix_pack(unsigned lo, unsigned hi, int be, unsigned sign) {
+  const unsigned long long t = fix_words(lo, hi) + 0x200ULL;
+  const unsigned th = (unsigned)(t >> 32);
+  return fix_from_bits((long long)fix_words(fix_shr_lo((unsigned)t, th, 10),
+                                            ((th >> 10) + ((unsigned)be << 20)) | sign));
+}
+
+// m 2^e rounded to nearest, 2^32 <= m < 2^63; the result has to be a normal double.
+MG_HD double fix_double_top(unsigned long long m, int e, unsigned sign = 0) {
+  const unsigned lo = (unsigned)m, hi = (unsigned)(m >> 32);
+  const int s = fix_clz32(hi) - 1;  // to bit 62
+  return fix_pack(lo << s, fix_shl_hi(lo, hi, s), e - s + (10 + 52 + 1023 - 1), sign);
+}
+
+// The same for any m < 2^63.
+MG_HD double fix_double(unsigned long long m, int e, unsigned sign = 0) {
+  const bool up = (m >> 32) == 0;
+  const double r = fix_double_top(up ? m << 31 : m, up ? e - 31 : e, sign);
+  return m == 0 ? 0.0 : r;
+}
+
+MG_HD double fix_signed(long long v, const FixRef& r) {
+  const unsigned n = (unsigned)(fix_hi(v) >> 31);
+  const unsigned long long f = fix_words(n, n);
+  return fix_double(((unsigned long long)v ^ f) - f, r.ue,
+                    (n ^ (r.neg ? 0xffffffffu : 0u)) & 0x80000000u);
+}
+
+// Sum a^2 + (3/8) sum c^2 = N 2^(64 - 2 sh) of integers below 2^62 (top: their high words
+// or-ed, signs removed): each value is shifted so that the largest lies in [2^61, 2^62)
+// and split as h 2^32 + l with -2^31 <= l < 2^31; h^2 and h l are exact, l^2 (a quarter
+// of a unit of N at most) is left out.
+MG_HD unsigned long long fix_quad(const long long (&a)[3], const long long (&c)[3], int& sh,
+                                  unsigned& top) {
+  top = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int ha = fix_hi(a[k]), hc = fix_hi(c[k]);
+    top |= (unsigned)(ha ^ (ha >> 31));
+    top |= (unsigned)(hc ^ (hc >> 31));
+  }
+  sh = fix_clz32(top) - 2;
+  auto form = [&](const long long (&v)[3]) {
+    long long hh = 0, hl = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const unsigned lo = (unsigned)v[k], xl = lo << sh;
+      const int h = (int)(fix_shl_hi(lo, (unsigned)fix_hi(v[k]), sh) + (xl >> 31));
+      hh += (long long)h * h;
+      hl += (long long)h * (int)xl;
+    }
+    return (unsigned long long)(hh + (hl >> 31));  // never negative
+  };
+  return form(a) + ((3ULL * form(c)) >> 3);
+}
+
+// sqrt(q) of a normal q > 0.  With Q = q scaled by an even power of two into
+// [2^60, 2^62): s0 = Q rsqrt(Q) in FP32 as an integer (error 2^-22 of s0), then twice
+// the residual Q - s^2 over 2 s0, in FP32: 2^-43, then below 2^-60.
+MG_HD double sqrt_fix_normal(double q) {
+  const long long b = fix_bits(q);
+  const unsigned lo = (unsigned)b, hi = (unsigned)(b >> 32);
+  const int e = (int)(hi >> 20);
+  const int odd = (e & 1) ^ 1;  // of the unbiased exponent
+  const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+  const unsigned long long Q = fix_words(lo << (8 + odd), fix_shl_hi(lo, mh, 8 + odd));
+  const float f = fix_float((fix_shl_hi(lo, hi, 3) & 0x7fffffu) + 0x3f800000u +
+                            ((unsigned)odd << 23));  // Q / 2^60 cut to 24 bits
+  const float y = fix_rsqrt(f);
+  const int s0 = fix_rint(f * y * 1073741824.f);
+  const long long r0 = (long long)Q - (long long)s0 * s0;
+  const unsigned r0l = (unsigned)r0, r0h = (unsigned)(r0 >> 32);
+  // d0: units of 2^-16; the residual left is (2^32 r0 - 2^17 s0 d0 - d0^2)
+  const int d0 = fix_rint((float)(int)fix_shr_lo(r0l, r0h, 12) * (y * 0.125f));
+  const long long u = (long long)fix_words(r0l << 15, fix_shl_hi(r0l, r0h, 15)) -
+                      (long long)s0 * d0;
+  const long long dd = (long long)d0 * d0;
+  const int r1 = (int)(fix_shr_lo((unsigned)u, (unsigned)(u >> 32), 5) -
+                       fix_shr_lo((unsigned)dd, (unsigned)(dd >> 32), 22));
+  const int d1 = fix_rint((float)r1 * (y * 0.001953125f));  // units of 2^-32
+  const long long t = (long long)d0 * 65536 + d1;
+  // s0 2^32 + t in [2^62, 2^63)
+  return fix_pack((unsigned)t, (unsigned)s0 + (unsigned)(t >> 32),
+                  ((e - 1023 - odd) >> 1) + 1022, 0);
+}
+
+}  // namespace mg

@@ -5,12 +5,14 @@
 // solve in one CTA, density restriction, gauge fix and the force output.
 //
 // Every kernel works on dense n^3 arrays, x fastest (idx = i + n(j + n k)), with
-// periodic wrap.  They are FP64-ALU bound on GB300 (about 35-45 FP64 operations
-// per cell against 24 bytes of traffic), so they favour a low FP64 instruction
-// count over memory tiling.
+// periodic wrap.  In FP64 they would be bound by GB300's narrow FP64 pipe (about 35-45
+// FP64 operations per cell against 24 bytes of traffic); the colour stages therefore do
+// the same arithmetic in integers (mg_fix64.cuh), the large levels in tiles
+// (mg_tile64.cuh), and the others favour a low FP64 instruction count.
 #include "mg_common.cuh"
 #include "mg_internal.h"
 #include "mg_bodies64.cuh"
+#include "mg_tile64.cuh"
 
 namespace mg {
 
@@ -20,13 +22,39 @@ namespace mg {
 // in the 19-point stencil), so the cells of one colour update independently
 // and each update is the exact Newton step of Sec. III.B.
 // ---------------------------------------------------------------------------
+// A warp takes a block of 8 x 2 x 2 of the colour's cells (x, y, z), a CTA warps / 2 of
+// them along x on each of two pairs of planes: a compact block mostly lies in one binade
+// of the field, which is the cheapest path of fix_align.
 __global__ void __launch_bounds__(256) k_smooth_colour64(int n, double* __restrict__ phi,
                                                          const double* __restrict__ src,
                                                          const double* __restrict__ f,
                                                          const LevelScalars* __restrict__ sc,
                                                          OpConst64 c, int colour) {
   PdlScope pdl_scope;
-  b_smooth_colour64(n, phi, src, f, sc, c, colour, blockIdx.x);
+  __shared__ double s_c;
+  if (threadIdx.x == 0) s_c = smooth_scalar64(sc, c);
+  __syncthreads();
+  const int hn = n >> 1;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int m = ((int)blockIdx.x * (int)(blockDim.x >> 6) + (w >> 1)) * 8 + (lane & 7);
+  const int jj = (int)blockIdx.y * 2 + ((lane >> 3) & 1);
+  const int k = (int)blockIdx.z * 4 + (w & 1) * 2 + (lane >> 4);
+  if (m >= hn || jj >= hn || k >= n) return;
+  cell_smooth64_at(n, phi, src, f, s_c, c, 2 * m + ((colour ^ k) & 1),
+                   2 * jj + (((colour >> 1) ^ k) & 1), k);
+}
+
+// The same for levels of many tiles.
+template <bool F>
+__global__ void __launch_bounds__(256, 4) k_smooth_tile64(int n, double* __restrict__ phi,
+                                                          const double* __restrict__ src,
+                                                          const double* __restrict__ f,
+                                                          const LevelScalars* __restrict__ sc,
+                                                          OpConst64 c, int colour) {
+  PdlScope pdl_scope;
+  __shared__ TileShared S;
+  b_smooth_tile64<F>(n, phi, src, f, sc, c, colour, (int)blockIdx.x * kTileX,
+                     (int)blockIdx.y * kTileY, (int)blockIdx.z * kTileZ, S);
 }
 
 // d = L^h phi - f with block partial norms.
@@ -276,15 +304,22 @@ int tpb_for(long long items) {
 
 void launch_smooth64(cudaStream_t st, int n, double* phi, const double* src, const double* f,
                      const LevelScalars* sc, const OpConst64& c, int sweeps, EventPairs* timer) {
-  const long long per = (long long)(n / 2) * (n / 2) * n;
-  const int tpb = tpb_for(per);
+  const int hn = n / 2;
+  const unsigned tpb = (unsigned)tpb_for((long long)hn * hn * n);
+  const unsigned bx = tpb / 8;  // cells of the colour along x per CTA
+  const dim3 grid((hn + bx - 1) / bx, (hn + 1) / 2, (n + 3) / 4);
+  const bool tiles = n >= kTileMinSide && c.mode != OP_GENW;
   for (int s = 0; s < sweeps; ++s)
     for (int colour = 0; colour < 4; ++colour) {
       // an event between two launches removes their programmatic overlap, so the
       // sampled mode brackets one colour stage per call
       const bool timed = timer && (!timer->first_only || (s == 0 && colour == 0));
       if (timed) timer->begin(st);
-      launch_k(k_smooth_colour64, blocks_for(per, tpb), tpb, 0, st, n, phi, src, f, sc, c, colour);
+      if (tiles)
+        launch_k(f ? k_smooth_tile64<true> : k_smooth_tile64<false>,
+                 tile_grid(n), 256, 0, st, n, phi, src, f, sc, c, colour);
+      else
+        launch_k(k_smooth_colour64, grid, tpb, 0, st, n, phi, src, f, sc, c, colour);
       if (timed) timer->end(st);
     }
   count_launches(4LL * sweeps);

@@ -32,10 +32,10 @@ void set_error(const std::string& msg);
 // may be scheduled while its predecessor in the stream finishes.  Every kernel
 // launched this way opens a PdlScope before touching memory.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_k(void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem,
+inline cudaError_t launch_k(void (*k)(KArgs...), dim3 grid, unsigned block, size_t smem,
                             cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
