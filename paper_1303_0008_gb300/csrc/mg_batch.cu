@@ -13,6 +13,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "mg_bodies32.cuh"
@@ -64,21 +65,37 @@ __device__ __forceinline__ const BItem& find_item(const BItem* __restrict__ item
   return items[lo];
 }
 
+// Origin of tile blk of an n^3 level, in the order of a launch over tile_grid.
+__device__ __forceinline__ int3 tile_origin(int n, long long blk) {
+  const dim3 g = tile_grid(n);
+  const unsigned b = (unsigned)blk, r = b / g.x;
+  return make_int3((int)(b - r * g.x) * kTileX, (int)(r % g.y) * kTileY, (int)(r / g.y) * kTileZ);
+}
+
+// run(f, lin) with both flags as types.
+template <typename Run>
+__device__ __forceinline__ void pick(bool f, bool lin, Run run) {
+  using T = std::true_type;
+  using N = std::false_type;
+  if (lin)
+    f ? run(T{}, T{}) : run(N{}, T{});
+  else
+    f ? run(T{}, N{}) : run(N{}, N{});
+}
+
 // ---- FP64 stages ----
 __global__ void __launch_bounds__(256) kb_smooth64(const BItem* __restrict__ items, int count,
                                                    int colour) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
   __shared__ TileShared S;
-  if (it.n >= kTileMinSide) {
-    const dim3 g = tile_grid(it.n);
-    const unsigned b = (unsigned)blk, r = b / g.x;
-    const int x0 = (int)(b - r * g.x) * kTileX, y0 = (int)(r % g.y) * kTileY,
-              z0 = (int)(r / g.y) * kTileZ;
-    if (it.f)
-      b_smooth_tile64<true>(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, x0, y0, z0, S);
-    else
-      b_smooth_tile64<false>(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, x0, y0, z0, S);
+  if (smooth_in_tiles(it.n, it.op)) {
+    const int3 o = tile_origin(it.n, blk);
+    auto run = [&](auto f, auto lin) {
+      b_smooth_tile64<decltype(f)::value, decltype(lin)::value>(
+          it.n, it.phi, it.src, it.f, it.sc, it.op, colour, o.x, o.y, o.z, S);
+    };
+    pick(it.f != nullptr, it.op.mode == OP_LINEAR, run);
     return;
   }
   b_smooth_colour64(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, blk);
@@ -88,6 +105,18 @@ __global__ void __launch_bounds__(256) kb_residual_restrict64(const BItem* __res
                                                               int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
+  __shared__ TileShared S;
+  if (in_tiles(it.n, it.op)) {
+    const int3 o = tile_origin(it.n, blk);
+    Partial p;
+    auto run = [&](auto f, auto lin) {
+      p = b_residual_restrict_tile64<decltype(f)::value, decltype(lin)::value>(
+          it.n, it.phi, it.src, it.f, it.op, it.cphi, it.cphihat, it.cf, o.x, o.y, o.z, S);
+    };
+    pick(it.f != nullptr, it.op.mode == OP_LINEAR, run);
+    if (threadIdx.x == 0) it.part[blk] = p;
+    return;
+  }
   b_residual_restrict64(it.n, it.phi, it.src, it.f, it.op, it.cphi, it.cphihat, it.cf, it.part,
                         blk);
 }
@@ -104,7 +133,9 @@ __global__ void __launch_bounds__(256) kb_finalize(const BItem* __restrict__ ite
   // cells; 2: the hand-off's, one per 256 kHandoffCells cells
   const long long work = mode == 0 ? cells / 8 : cells;
   const int per = mode == 2 ? 256 * kHandoffCells : 256;
-  const int nparts = (int)((work + per - 1) / per);
+  // the FP64 kernels of a level in tiles leave one partial per tile
+  const int nparts = !use32 && in_tiles(it.n, it.op) ? (int)tile_count(it.n)
+                                                     : (int)((work + per - 1) / per);
   LevelScalars* sc = use32 ? it.sc32 : it.sc;
   b_finalize(it.part, nparts, (double)cells, 1, sc, 0);
   if (threadIdx.x == 0) {
@@ -116,6 +147,17 @@ __global__ void __launch_bounds__(256) kb_finalize(const BItem* __restrict__ ite
 __global__ void __launch_bounds__(256) kb_fas_rhs64(const BItem* __restrict__ items, int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
+  __shared__ TileShared S;
+  if (in_tiles(it.n / 2, it.cop)) {
+    const int3 o = tile_origin(it.n / 2, blk);
+    if (it.cop.mode == OP_LINEAR)
+      b_fas_rhs_tile64<true>(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, o.x, o.y,
+                             o.z, S);
+    else
+      b_fas_rhs_tile64<false>(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, o.x, o.y,
+                              o.z, S);
+    return;
+  }
   b_fas_rhs64(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, blk);
 }
 
@@ -135,8 +177,18 @@ __global__ void __launch_bounds__(256) kb_coarsest64(const BItem* __restrict__ i
 __global__ void __launch_bounds__(256) kb_handoff64(const BItem* __restrict__ items, int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
-  b_residual_handoff64(it.n, it.phi, it.src, it.op, it.sc, it.rhs, it.q0, it.phi0, it.e, it.part,
-                       blk);
+  __shared__ TileShared S;
+  const Handoff out{it.rhs, it.q0, it.phi0, it.e, nullptr, nullptr};
+  if (in_tiles(it.n, it.op)) {
+    const int3 o = tile_origin(it.n, blk);
+    const Partial p =
+        it.op.mode == OP_LINEAR
+            ? b_handoff_tile64<true>(it.n, it.phi, it.src, it.op, it.sc, out, o.x, o.y, o.z, S)
+            : b_handoff_tile64<false>(it.n, it.phi, it.src, it.op, it.sc, out, o.x, o.y, o.z, S);
+    if (threadIdx.x == 0) it.part[blk] = p;
+    return;
+  }
+  b_residual_handoff64(it.n, it.phi, it.src, it.op, it.sc, out, it.part, blk);
 }
 
 __global__ void __launch_bounds__(256) kb_update64(const BItem* __restrict__ items, int count) {
@@ -196,22 +248,32 @@ __global__ void __launch_bounds__(256) kb_coarsest_corr32(const BItem* __restric
 // Host side
 // ---------------------------------------------------------------------------
 // T_HAND: the outer residual hand-off, kHandoffCells cells per thread
-// T_SM64: the FP64 colour stages, in tiles from kTileMinSide on
-enum ListType { T_SMOOTH = 0, T_RR, T_CELL, T_CCELL, T_ONE, T_HAND, T_SM64, T_NTYPES };
+// T_SM64, T_RR64, T_CCELL64: the FP64 colour stages, residual restrictions and right-hand
+// sides (of the level below), and T_HAND: in tiles from kTileMinSide on
+enum ListType {
+  T_SMOOTH = 0, T_RR, T_CELL, T_CCELL, T_ONE, T_HAND, T_SM64, T_RR64, T_CCELL64, T_NTYPES
+};
 
-static long long blocks_of(ListType t, int n) {
+static long long blocks_of(ListType t, const BItem& it) {
+  const int n = it.n;
   const long long cells = (long long)n * n * n;
   switch (t) {
+    case T_SM64:
+      if (smooth_in_tiles(n, it.op)) return tile_count(n);
+      return (cells / 4 + 255) / 256;
     case T_SMOOTH: return (cells / 4 + 255) / 256;
-    case T_SM64: {
-      if (n < kTileMinSide) return (cells / 4 + 255) / 256;
-      const dim3 g = tile_grid(n);
-      return (long long)g.x * g.y * g.z;
-    }
+    case T_RR64:
+      if (in_tiles(n, it.op)) return tile_count(n);
+      return (cells / 8 + 255) / 256;
     case T_RR: return (cells / 8 + 255) / 256;
     case T_CELL: return (cells + 255) / 256;
+    case T_CCELL64:
+      if (in_tiles(n / 2, it.cop)) return tile_count(n / 2);
+      return (cells / 8 + 255) / 256;
     case T_CCELL: return (cells / 8 + 255) / 256;
-    case T_HAND: return (cells + 256 * kHandoffCells - 1) / (256 * kHandoffCells);
+    case T_HAND:
+      if (in_tiles(n, it.op)) return tile_count(n);
+      return (cells + 256 * kHandoffCells - 1) / (256 * kHandoffCells);
     default: return 1;
   }
 }
@@ -362,7 +424,7 @@ static mg_status build_lists(mg_grid* g, const SolveParams& P) {
           if (!ok) continue;
           BItem it = make_item(g, P, s, l);
           it.block0 = (int)blocks;
-          blocks += blocks_of((ListType)t, it.n);
+          blocks += blocks_of((ListType)t, it);
           maxn = std::max(maxn, it.n);
           items.push_back(it);
         }
@@ -415,18 +477,18 @@ struct BatchCycle {
   }
   void part_a64() const {
     smooth64(0, o->nu_pre);
-    launch(L(0, T_RR, P_DESC), 256, kb_residual_restrict64);
+    launch(L(0, T_RR64, P_DESC), 256, kb_residual_restrict64);
     finalize(0, T_RR, 0, 0, 0);
     cudaMemcpyAsync(bs->h_out, bs->d_out, sizeof(LevelScalars) * g->domains.size(),
                     cudaMemcpyDeviceToHost, st);
   }
   void part_b64() const {
-    launch(L(0, T_CCELL, P_DESC), 256, kb_fas_rhs64);
+    launch(L(0, T_CCELL64, P_DESC), 256, kb_fas_rhs64);
     for (int l = 1; l < bs->lmax - 1; ++l) {
       smooth64(l, o->nu_pre);
-      launch(L(l, T_RR, P_DESC), 256, kb_residual_restrict64);
+      launch(L(l, T_RR64, P_DESC), 256, kb_residual_restrict64);
       finalize(l, T_RR, 0, 0, 0);
-      launch(L(l, T_CCELL, P_DESC), 256, kb_fas_rhs64);
+      launch(L(l, T_CCELL64, P_DESC), 256, kb_fas_rhs64);
     }
     const size_t smem = 3 * sizeof(double) * (size_t)bs->coarsest.maxn * bs->coarsest.maxn *
                         bs->coarsest.maxn;

@@ -2,7 +2,8 @@
 // mg_bodies64.cuh for the convention).
 #pragma once
 
-#include "mg_common.cuh"
+#include "mg_bodies64.cuh"
+#include "mg_tile64.cuh"
 
 namespace mg {
 
@@ -80,10 +81,6 @@ __device__ __forceinline__ float2 dD2(const Stencil2& se, const Stencil2& sp, fl
   return make_float2(root_change32(q0.x, q1.x, du.x, c), root_change32(q0.y, q1.y, du.y, c));
 }
 
-// The FP64 residual of the outer defect correction and its hand-off to the FP32
-// inner problem.  Each thread takes kHandoffCells cells (a block covers
-// 256 kHandoffCells consecutive cells, coalesced per step), so the block's norm
-// reduction, about 15 FP64 warp instructions, is shared by several cells.
 // Index of cell (i,j,k) of an n^3 grid in colour order: the cells of colour
 // c = ((i+k)&1) + 2((j+k)&1) fill block c of n^3/4 entries, in the order in which
 // the threads of a colour stage visit them (x fastest, then y, then z), so that a
@@ -94,13 +91,36 @@ __device__ __forceinline__ long long colour_index(int i, int j, int k, int n) {
   return colour * (hn * hn * n) + ((long long)k * hn + (j >> 1)) * hn + (i >> 1);
 }
 
-// With q0c / gc (may be null) the hand-off also stores q0 and g in colour order
-// (colour_index) for the colour stages of the finest level.
-__device__ __forceinline__ void b_residual_handoff64(
-    int n, const double* __restrict__ phi, const double* __restrict__ src, OpConst64 c,
-    const LevelScalars* __restrict__ sc, float* __restrict__ g, float* __restrict__ q0,
-    float* __restrict__ phi0, float* __restrict__ e, Partial* __restrict__ partials,
-    long long blk, float* __restrict__ gc = nullptr, float* __restrict__ q0c = nullptr) {
+// The FP64 residual of the outer defect correction and its hand-off to the FP32
+// inner problem.  Each thread takes kHandoffCells cells (a block covers
+// 256 kHandoffCells consecutive cells, coalesced per step), so the block's norm
+// reduction, about 15 FP64 warp instructions, is shared by several cells.
+// Where the hand-off goes; with gc and q0c (may be null) g and q0 also in colour order
+// (colour_index), for the colour stages of the finest level.
+struct Handoff {
+  float *g, *q0, *phi0, *e, *gc, *q0c;
+  __device__ __forceinline__ void store(int n, int i, int j, int k, long long t, double phi,
+                                        double rhs, double q) const {
+    const float gv = fix_to_float(rhs), qv = fix_to_float(q);
+    g[t] = gv;
+    q0[t] = qv;
+    phi0[t] = fix_to_float(phi);
+    e[t] = 0.f;
+    if (gc) {
+      const long long ci = colour_index(i, j, k, n);
+      gc[ci] = gv;
+      q0c[ci] = qv;
+    }
+  }
+};
+
+__device__ __forceinline__ void b_residual_handoff64(int n, const double* __restrict__ phi,
+                                                     const double* __restrict__ src,
+                                                     const OpConst64& c,
+                                                     const LevelScalars* __restrict__ sc,
+                                                     const Handoff& out,
+                                                     Partial* __restrict__ partials,
+                                                     long long blk) {
   const long long cells = (long long)n * n * n;
   Partial p;
   partial_init(p);
@@ -111,40 +131,34 @@ __device__ __forceinline__ void b_residual_handoff64(
     if (t >= cells) break;
     int i, j, k;
     split3((unsigned)t, n, i, j, k);
-    const StencilT<double> s = gather_periodic(phi, i, j, k, n);
-    double q = 1.0, D;
-    bool guard = false;
-    if (c.mode == OP_LINEAR) {
-      D = src[t];
-    } else {
-      const double A2 = half_A(s);
-      const double B = fma(s.cxy, s.cxy, fma(s.cxz, s.cxz, s.cyz * s.cyz));
-      if (c.mode == OP_SQRT) {
-        q = fma(c.e1h, A2, fma(c.e2, B, src[t]));
-        D = fma(c.k2s, sqrt_clamped(q), -c.k2);
-      } else {
-        const double u = fma(c.c1h, A2, fma(c.c2, B, src[t]));
-        q = fma(c.c3, u, 1.0);
-        D = (q < 0.0) ? -c.k2 : (2.0 * u) / (1.0 + sqrt(q));
-      }
-      guard = neg_guard(q);
-    }
-    const double ctr = phi[t];
-    const double lap = (s.sx + s.sy + s.sz) - 6.0 * ctr;
-    const double d = fma(lap, c.inv_h2, -D);
+    double q;
+    bool guard;
+    const double d = cell_defect_fix64(phi, n, i, j, k, t, src[t], c, q, guard);
     partial_add(p, d, guard);
-    g[t] = (float)(lam - d);
-    q0[t] = (float)q;
-    phi0[t] = (float)ctr;
-    e[t] = 0.f;
-    if (gc) {
-      const long long ci = colour_index(i, j, k, n);
-      gc[ci] = (float)(lam - d);
-      q0c[ci] = (float)q;
-    }
+    out.store(n, i, j, k, t, phi[t], lam - d, q);
   }
   p = block_reduce(p);
   if (threadIdx.x == 0) partials[blk] = p;
+}
+
+// The same for a tile; its partial (thread 0).
+template <bool LIN>
+__device__ __forceinline__ Partial b_handoff_tile64(int n, const double* __restrict__ phi,
+                                                    const double* __restrict__ src,
+                                                    const OpConst64& c,
+                                                    const LevelScalars* __restrict__ sc,
+                                                    const Handoff& out, int x0, int y0, int z0,
+                                                    TileShared& S) {
+  Partial p;
+  partial_init(p);
+  const double lam = sc->lambda;
+  tile_defects<LIN>(
+      n, phi, c, x0, y0, z0, S, [&](int id) { return src[id]; },
+      [&](int id, int i, int j, int k, double d, double q, bool g) {
+        partial_add(p, d, g);
+        out.store(n, i, j, k, id, phi[id], lam - d, q);
+      });
+  return tile_reduce(p, S);
 }
 
 __device__ __forceinline__ void b_update64(long long cells, double* __restrict__ phi,

@@ -90,20 +90,35 @@ __device__ __forceinline__ void b_smooth_colour64(int n, double* __restrict__ ph
   cell_smooth64(n, phi, src, f, s_c, c, colour, (long long)blk * blockDim.x + threadIdx.x);
 }
 
-// The defect d = L(phi) - f of fine cell (i,j,k) (linear index id) and its guard
-// flag; ctr returns phi there.
+// The defect L(phi) of cell (i,j,k) (linear index id) without a right-hand side, its
+// discriminant (1 where the mode has none) and guard flag.
+__device__ __forceinline__ double cell_defect_fix64(const double* __restrict__ phi, int n, int i,
+                                                    int j, int k, long long id, double src,
+                                                    const OpConst64& c, double& q, bool& g) {
+  auto nbr = [&] { return nbr_offsets(i, j, k, n); };
+  if (c.mode == OP_GENW) {
+    const StencilT<double> s = gather_at(phi + id, nbr());
+    q = 1.0;
+    const double D = root_Dc(s, phi[id], src, c, g);
+    return fma((s.sx + s.sy + s.sz) - 6.0 * phi[id], c.inv_h2, -D);
+  }
+  long long b[19];
+  gather_bits(phi + id, nbr(), b);
+  double lap, M;
+  stencil_forms(phi + id, nbr, b, c.mode != OP_LINEAR, lap, M);
+  return fma(lap, c.inv_h2, -root_of_M(M, src, c, q, g));
+}
+
+// The defect d = L(phi) - f of fine cell (i,j,k) and its guard flag; ctr returns phi there.
 __device__ __forceinline__ double fine_defect64(int nf, const double* __restrict__ phi,
                                                const double* __restrict__ src,
                                                const double* __restrict__ f,
                                                const OpConst64& c, int i, int j, int k,
                                                long long id, double& ctr, bool& g) {
-  const StencilT<double> s = gather_periodic(phi, i, j, k, nf);
   ctr = phi[id];
-  const double D = root_Dc(s, ctr, src[id], c, g);
-  const double lap = (s.sx + s.sy + s.sz) - 6.0 * ctr;
-  double d = fma(lap, c.inv_h2, -D);
-  if (f) d -= f[id];
-  return d;
+  double q;
+  const double d = cell_defect_fix64(phi, nf, i, j, k, id, src[id], c, q, g);
+  return f ? d - f[id] : d;
 }
 
 __device__ __forceinline__ void b_residual_restrict64(
@@ -262,11 +277,9 @@ __device__ __forceinline__ void cell_fas_rhs64(int nc, const double* __restrict_
   if (t >= cells) return;
   int i, j, k;
   split3((unsigned)t, nc, i, j, k);
-  const StencilT<double> s = gather_periodic(phi_c, i, j, k, nc);
+  double q;
   bool g;
-  const double D = root_Dc(s, phi_c[t], src_c[t], c, g);
-  const double lap = (s.sx + s.sy + s.sz) - 6.0 * phi_c[t];
-  const double L = fma(lap, c.inv_h2, -D);
+  const double L = cell_defect_fix64(phi_c, nc, i, j, k, t, src_c[t], c, q, g);
   f_c[t] = L - f_c[t] + lam_f;
 }
 

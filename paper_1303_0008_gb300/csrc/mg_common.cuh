@@ -296,8 +296,7 @@ __device__ __forceinline__ void stencil_forms(const double* at, Nbr nbr, long lo
 static __device__ __noinline__ double sqrt_clamped_rare(double q) { return sqrt_clamped(q); }
 
 __device__ __forceinline__ double sqrt_clamped_fix(double q) {
-  const unsigned e = (unsigned)(__double_as_longlong(q) >> 52);  // sign and exponent
-  return e - 1u < 2046u ? sqrt_fix_normal(q) : sqrt_clamped_rare(q);
+  return fix_normal(q) ? sqrt_fix_normal(q) : sqrt_clamped_rare(q);
 }
 
 // The root D of Eq. two_branch from M (stencil_forms) and the source term; q is the

@@ -10,7 +10,7 @@
 //               no conversion at all: their bit patterns differ by exactly the
 //               differences of their significands.  Values of one sign and near
 //               binades are shifted up, exactly; others are shifted to the largest
-//               exponent, with 7 more bits below.
+//               exponent, with 6 or 7 more bits below.
 //   sums        exact (FP64 rounds each to half a unit in the last place of the field).
 //   fix_quad    the quadratic form of Sigma_d as a 62-bit integer, error below 2^-53.
 //   sqrt_fix    square root to about 2^-61 from the FP32 reciprocal square root and two
@@ -128,8 +128,12 @@ constexpr int kFixMinExp = 640, kFixMaxExp = 1470;
 
 // Replace the bit patterns b[] by integers of one unit; false when the values have no
 // such form (b is then unchanged).
+//
+// NV = 18 leaves the largest below 2^60, for sums of six; NV = 19 (with the centre, of
+// which six are subtracted) below 2^59.
 template <int NV>
 MG_HD bool fix_align(long long (&b)[NV], FixRef& r) {
+  constexpr int kUp = NV == 19 ? 6 : 7;  // bits above a significand
   const int h0 = fix_hi(b[0]);
   int diff = 0;
 #pragma unroll
@@ -149,9 +153,9 @@ MG_HD bool fix_align(long long (&b)[NV], FixRef& r) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       d[k] = ((unsigned)fix_hi(b[k]) >> 20) - lo;
-      far |= d[k];
+      far = d[k] > far ? d[k] : far;
     }
-    if (far <= 7u) {
+    if (far <= (unsigned)kUp) {
 #pragma unroll
       for (int k = 0; k < NV; ++k)
         b[k] = (long long)((((unsigned long long)b[k] & 0xfffffffffffffULL) | 0x10000000000000ULL)
@@ -176,11 +180,11 @@ MG_HD bool fix_align(long long (&b)[NV], FixRef& r) {
     d = d > 63 ? 63 : d;
     const long long s = b[k] >> 63;
     const unsigned long long m =
-        (((unsigned long long)b[k] & 0xfffffffffffffULL) | 0x10000000000000ULL) << 7;
+        (((unsigned long long)b[k] & 0xfffffffffffffULL) | 0x10000000000000ULL) << kUp;
     b[k] = (long long)((m >> d) ^ (unsigned long long)s) - s;
   }
   r.off6 = 0;
-  r.ue = (em >> 20) - 1082;
+  r.ue = (em >> 20) - 1075 - kUp;
   r.neg = false;
   return true;
 }
@@ -243,6 +247,11 @@ MG_HD unsigned long long fix_quad(const long long (&a)[3], const long long (&c)[
   return form(a) + ((3ULL * form(c)) >> 3);
 }
 
+// Whether q is a normal double above 0.
+MG_HD bool fix_normal(double q) {
+  return ((unsigned)(fix_bits(q) >> 32) >> 20) - 1u < 2046u;
+}
+
 // sqrt(q) of a normal q > 0.  With Q = q scaled by an even power of two into
 // [2^60, 2^62): s0 = Q rsqrt(Q) in FP32 as an integer (error 2^-22 of s0), then twice
 // the residual Q - s^2 over 2 s0, in FP32: 2^-43, then below 2^-60.
@@ -272,5 +281,20 @@ MG_HD double sqrt_fix_normal(double q) {
   return fix_pack((unsigned)t, (unsigned)s0 + (unsigned)(t >> 32),
                   ((e - 1023 - odd) >> 1) + 1022, 0);
 }
+
+#ifdef __CUDACC__
+static __device__ __noinline__ float fix_to_float_rare(double x) { return (float)x; }
+
+// (float)x, rounded to nearest even: the conversion instruction runs on the FP64 pipe.
+__device__ __forceinline__ float fix_to_float(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const unsigned h = ((unsigned)hi & 0x7fffffffu) - 0x38000000u;  // exponent bias 1023 -> 127
+  if (h - 0x00100000u >= 0x0fe00000u) return fix_to_float_rare(x);  // not a normal float
+  unsigned r = __funnelshift_l(lo, h, 3);
+  r += ((lo << 3) + (r & 1u)) > 0x80000000u ? 1u : 0u;
+  return __uint_as_float(r | ((unsigned)hi & 0x80000000u));
+}
+#endif
 
 }  // namespace mg

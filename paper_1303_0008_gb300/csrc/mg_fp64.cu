@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(256) k_smooth_colour64(int n, double* __restri
 }
 
 // The same for levels of many tiles.
-template <bool F>
+template <bool F, bool LIN>
 __global__ void __launch_bounds__(256, 4) k_smooth_tile64(int n, double* __restrict__ phi,
                                                           const double* __restrict__ src,
                                                           const double* __restrict__ f,
@@ -53,8 +53,8 @@ __global__ void __launch_bounds__(256, 4) k_smooth_tile64(int n, double* __restr
                                                           OpConst64 c, int colour) {
   PdlScope pdl_scope;
   __shared__ TileShared S;
-  b_smooth_tile64<F>(n, phi, src, f, sc, c, colour, (int)blockIdx.x * kTileX,
-                     (int)blockIdx.y * kTileY, (int)blockIdx.z * kTileZ, S);
+  b_smooth_tile64<F, LIN>(n, phi, src, f, sc, c, colour, (int)blockIdx.x * kTileX,
+                          (int)blockIdx.y * kTileY, (int)blockIdx.z * kTileZ, S);
 }
 
 // d = L^h phi - f with block partial norms.
@@ -69,20 +69,40 @@ __global__ void __launch_bounds__(256) k_residual64(int n, const double* __restr
   Partial p;
   partial_init(p);
   if (t < cells) {
-    const int i = (int)(t % n);
-    const int j = (int)((t / n) % n);
-    const int k = (int)(t / ((long long)n * n));
-    const StencilT<double> s = gather_periodic(phi, i, j, k, n);
+    int i, j, k;
+    split3((unsigned)t, n, i, j, k);
     bool g;
-    const double D = root_Dc(s, phi[t], src[t], c, g);
-    const double lap = (s.sx + s.sy + s.sz) - 6.0 * phi[t];
-    double d = fma(lap, c.inv_h2, -D);
-    if (f) d -= f[t];
+    double ctr;
+    const double d = fine_defect64(n, phi, src, f, c, i, j, k, t, ctr, g);
     if (dout) dout[t] = d;
     partial_add(p, d, g);
   }
   p = block_reduce(p);
   if (threadIdx.x == 0) partials[blockIdx.x] = p;
+}
+
+// The same for levels of many tiles, one partial per tile.
+template <bool LIN>
+__global__ void __launch_bounds__(256, 3) k_residual_tile64(int n, const double* __restrict__ phi,
+                                                            const double* __restrict__ src,
+                                                            const double* __restrict__ f,
+                                                            double* __restrict__ dout,
+                                                            OpConst64 c,
+                                                            Partial* __restrict__ partials) {
+  PdlScope pdl_scope;
+  __shared__ TileShared S;
+  Partial p;
+  partial_init(p);
+  tile_defects<LIN>(
+      n, phi, c, (int)blockIdx.x * kTileX, (int)blockIdx.y * kTileY, (int)blockIdx.z * kTileZ, S,
+      [&](int id) { return src[id]; },
+      [&](int id, int, int, int, double d, double, bool g) {
+        if (f) d -= f[id];
+        if (dout) dout[id] = d;
+        partial_add(p, d, g);
+      });
+  p = tile_reduce(p, S);
+  if (threadIdx.x == 0) partials[tile_index()] = p;
 }
 
 // Residual of the 8 children of each coarse cell, averaged (full weighting),
@@ -93,6 +113,21 @@ __global__ void __launch_bounds__(256) k_residual_restrict64(
     double* __restrict__ phihat_c, double* __restrict__ rd_c, Partial* __restrict__ partials) {
   PdlScope pdl_scope;
   b_residual_restrict64(nf, phi, src, f, c, phi_c, phihat_c, rd_c, partials, blockIdx.x);
+}
+
+// The same for levels of many tiles, one partial per tile.
+template <bool F, bool LIN>
+__global__ void __launch_bounds__(256, 2) k_residual_restrict_tile64(
+    int nf, const double* __restrict__ phi, const double* __restrict__ src,
+    const double* __restrict__ f, OpConst64 c, double* __restrict__ phi_c,
+    double* __restrict__ phihat_c, double* __restrict__ rd_c, Partial* __restrict__ partials) {
+  PdlScope pdl_scope;
+  __shared__ TileShared S;
+  const Partial p = b_residual_restrict_tile64<F, LIN>(nf, phi, src, f, c, phi_c, phihat_c, rd_c,
+                                                  (int)blockIdx.x * kTileX,
+                                                  (int)blockIdx.y * kTileY,
+                                                  (int)blockIdx.z * kTileZ, S);
+  if (threadIdx.x == 0) partials[tile_index()] = p;
 }
 
 // The same residual restriction in two launches, for levels whose coarse cells
@@ -149,6 +184,19 @@ __global__ void __launch_bounds__(256) k_fas_rhs64(int nc, const double* __restr
                                                    LevelScalars* __restrict__ coarse_sc) {
   PdlScope pdl_scope;
   b_fas_rhs64(nc, phi_c, src_c, f_c, c, fine_sc, coarse_sc, blockIdx.x);
+}
+
+// The same for levels of many tiles.
+template <bool LIN>
+__global__ void __launch_bounds__(256, 3) k_fas_rhs_tile64(int nc, const double* __restrict__ phi_c,
+                                                           const double* __restrict__ src_c,
+                                                           double* __restrict__ f_c, OpConst64 c,
+                                                           const LevelScalars* __restrict__ fine_sc,
+                                                           LevelScalars* __restrict__ coarse_sc) {
+  PdlScope pdl_scope;
+  __shared__ TileShared S;
+  b_fas_rhs_tile64<LIN>(nc, phi_c, src_c, f_c, c, fine_sc, coarse_sc, (int)blockIdx.x * kTileX,
+                   (int)blockIdx.y * kTileY, (int)blockIdx.z * kTileZ, S);
 }
 
 // phi^h += P(phi^H - R phi^h): cell-centred trilinear, per axis 3/4 on the parent
@@ -308,7 +356,9 @@ void launch_smooth64(cudaStream_t st, int n, double* phi, const double* src, con
   const unsigned tpb = (unsigned)tpb_for((long long)hn * hn * n);
   const unsigned bx = tpb / 8;  // cells of the colour along x per CTA
   const dim3 grid((hn + bx - 1) / bx, (hn + 1) / 2, (n + 3) / 4);
-  const bool tiles = n >= kTileMinSide && c.mode != OP_GENW;
+  const bool tiles = smooth_in_tiles(n, c), lin = c.mode == OP_LINEAR;
+  auto tile_kernel = lin ? (f ? k_smooth_tile64<true, true> : k_smooth_tile64<false, true>)
+                         : (f ? k_smooth_tile64<true, false> : k_smooth_tile64<false, false>);
   for (int s = 0; s < sweeps; ++s)
     for (int colour = 0; colour < 4; ++colour) {
       // an event between two launches removes their programmatic overlap, so the
@@ -316,8 +366,7 @@ void launch_smooth64(cudaStream_t st, int n, double* phi, const double* src, con
       const bool timed = timer && (!timer->first_only || (s == 0 && colour == 0));
       if (timed) timer->begin(st);
       if (tiles)
-        launch_k(f ? k_smooth_tile64<true> : k_smooth_tile64<false>,
-                 tile_grid(n), 256, 0, st, n, phi, src, f, sc, c, colour);
+        launch_k(tile_kernel, tile_grid(n), 256, 0, st, n, phi, src, f, sc, c, colour);
       else
         launch_k(k_smooth_colour64, grid, tpb, 0, st, n, phi, src, f, sc, c, colour);
       if (timed) timer->end(st);
@@ -331,8 +380,12 @@ void launch_residual64(cudaStream_t st, int n, const double* phi, const double* 
                        const double* f, double* dout, const OpConst64& c, Partial* partials,
                        LevelScalars* sc, int periodic) {
   const long long cells = (long long)n * n * n;
-  const unsigned nb = blocks_for(cells, 256);
-  launch_k(k_residual64, nb, 256, 0, st, n, phi, src, f, dout, c, partials);
+  const bool tiles = in_tiles(n, c);
+  const unsigned nb = tiles ? tile_count(n) : blocks_for(cells, 256);
+  if (tiles)
+    launch_k(c.mode == OP_LINEAR ? k_residual_tile64<true> : k_residual_tile64<false>, tile_grid(n), 256, 0, st, n, phi, src, f, dout, c, partials);
+  else
+    launch_k(k_residual64, nb, 256, 0, st, n, phi, src, f, dout, c, partials);
   launch_k(k_finalize, 1, 256, 0, st, partials, (int)nb, (double)cells, periodic, sc);
   count_launches(2);
 }
@@ -343,8 +396,16 @@ void launch_residual_restrict64(cudaStream_t st, int nf, const double* phi, cons
                                 LevelScalars* sc, double* def, unsigned char* guard) {
   const long long fcells = (long long)nf * nf * nf;
   const long long ccells = fcells / 8;
-  const unsigned nb = blocks_for(ccells, 256);
-  if (def && guard && fcells <= kTwoStepMaxFine) {
+  const bool tiles = in_tiles(nf, c);
+  const unsigned nb = tiles ? tile_count(nf) : blocks_for(ccells, 256);
+  if (tiles) {
+    const bool lin = c.mode == OP_LINEAR;
+    launch_k(lin ? (f ? k_residual_restrict_tile64<true, true>
+                      : k_residual_restrict_tile64<false, true>)
+                 : (f ? k_residual_restrict_tile64<true, false>
+                      : k_residual_restrict_tile64<false, false>),
+             tile_grid(nf), 256, 0, st, nf, phi, src, f, c, phi_c, phihat_c, rd_c, partials);
+  } else if (def && guard && fcells <= kTwoStepMaxFine) {
     const int tpb = tpb_for(fcells);
     launch_k(k_defect64, blocks_for(fcells, tpb), tpb, 0, st, nf, phi, src, f, c, def, guard);
     launch_k(k_restrict_defects64, nb, 256, 0, st, nf, phi, (const double*)def,
@@ -363,8 +424,12 @@ void launch_fas_rhs64(cudaStream_t st, int nc, const double* phi_c, const double
                       LevelScalars* coarse_sc) {
   const long long cells = (long long)nc * nc * nc;
   const int tpb = tpb_for(cells);
-  launch_k(k_fas_rhs64, blocks_for(cells, tpb), tpb, 0, st, nc, phi_c, src_c, f_c, c, fine_sc,
-           coarse_sc);
+  if (in_tiles(nc, c))
+    launch_k(c.mode == OP_LINEAR ? k_fas_rhs_tile64<true> : k_fas_rhs_tile64<false>, tile_grid(nc), 256, 0, st, nc, phi_c, src_c, f_c, c, fine_sc,
+             coarse_sc);
+  else
+    launch_k(k_fas_rhs64, blocks_for(cells, tpb), tpb, 0, st, nc, phi_c, src_c, f_c, c, fine_sc,
+             coarse_sc);
   count_launches(1);
 }
 

@@ -39,13 +39,29 @@ namespace mg {
 // ---------------------------------------------------------------------------
 // FP64 outer residual with the FP32 hand-off.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_residual_handoff64(
-    int n, const double* __restrict__ phi, const double* __restrict__ src, OpConst64 c,
-    const LevelScalars* __restrict__ sc, float* __restrict__ g, float* __restrict__ q0,
-    float* __restrict__ phi0, float* __restrict__ e, Partial* __restrict__ partials,
-    float* __restrict__ gc, float* __restrict__ q0c) {
+__global__ void __launch_bounds__(256) k_residual_handoff64(int n, const double* __restrict__ phi,
+                                                            const double* __restrict__ src,
+                                                            OpConst64 c,
+                                                            const LevelScalars* __restrict__ sc,
+                                                            Handoff out,
+                                                            Partial* __restrict__ partials) {
   PdlScope pdl_scope;
-  b_residual_handoff64(n, phi, src, c, sc, g, q0, phi0, e, partials, blockIdx.x, gc, q0c);
+  b_residual_handoff64(n, phi, src, c, sc, out, partials, blockIdx.x);
+}
+
+// The same for levels of many tiles, one partial per tile.
+template <bool LIN>
+__global__ void __launch_bounds__(256, 3) k_handoff_tile64(int n, const double* __restrict__ phi,
+                                                           const double* __restrict__ src,
+                                                           OpConst64 c,
+                                                           const LevelScalars* __restrict__ sc,
+                                                           Handoff out,
+                                                           Partial* __restrict__ partials) {
+  PdlScope pdl_scope;
+  __shared__ TileShared S;
+  const Partial p = b_handoff_tile64<LIN>(n, phi, src, c, sc, out, (int)blockIdx.x * kTileX,
+                                     (int)blockIdx.y * kTileY, (int)blockIdx.z * kTileZ, S);
+  if (threadIdx.x == 0) partials[tile_index()] = p;
 }
 
 // phi += e (FP64).
@@ -528,9 +544,15 @@ struct CycleMixed {
   // FP64 residual, FP32 hand-off, convergence scalars to the host.
   void part_a() const {
     Level& L = d->lv[0];
-    const unsigned nb = nblk(L.cells, 256 * kHandoffCells);
-    launch_k(k_residual_handoff64, nb, 256, 0, st, L.n, L.phi, L.src, ops[0], d->d_sc, L.rhs, L.q0,
-             L.phi0, L.e, d->d_part, L.rhsc, L.q0c);
+    const bool tiles = in_tiles(L.n, ops[0]);
+    const unsigned nb = tiles ? tile_count(L.n) : nblk(L.cells, 256 * kHandoffCells);
+    const Handoff out{L.rhs, L.q0, L.phi0, L.e, L.rhsc, L.q0c};
+    if (tiles)
+      launch_k(ops[0].mode == OP_LINEAR ? k_handoff_tile64<true> : k_handoff_tile64<false>, tile_grid(L.n), 256, 0, st, L.n, L.phi, L.src, ops[0], d->d_sc,
+               out, d->d_part);
+    else
+      launch_k(k_residual_handoff64, nb, 256, 0, st, L.n, L.phi, L.src, ops[0], d->d_sc, out,
+               d->d_part);
     count_launches(1);
     launch_finalize(st, d->d_part, (int)nb, (double)L.cells, 1, d->d_sc);
     cudaMemcpyAsync(d->h_sc, d->d_sc, sizeof(LevelScalars), cudaMemcpyDeviceToHost, st);

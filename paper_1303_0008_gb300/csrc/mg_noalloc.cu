@@ -23,6 +23,7 @@
 
 #include "../../include/mg.h"
 #include "mg_internal.h"
+#include "mg_tile64.cuh"
 
 namespace mg {
 
@@ -50,20 +51,38 @@ __global__ void __launch_bounds__(kNoAllocThreads) k_residual64_noalloc(
   Partial p;
   partial_init(p);
   if (t < cells) {
-    const int i = (int)(t % n);
-    const int j = (int)((t / n) % n);
-    const int k = (int)(t / ((long long)n * n));
-    const StencilT<double> s = gather_periodic(phi, i, j, k, n);
+    int i, j, k;
+    split3((unsigned)t, n, i, j, k);
+    double q;
     bool g;
-    const double D = root_D(s, fma(a, delta[t], b), c, g);
-    const double lap = (s.sx + s.sy + s.sz) - 6.0 * phi[t];
-    double d = fma(lap, c.inv_h2, -D);
+    double d = cell_defect_fix64(phi, n, i, j, k, t, fma(a, delta[t], b), c, q, g);
     if (f) d -= f[t];
     if (dout) dout[t] = d;
     partial_add(p, d, g);
   }
   p = block_reduce(p);
   if (threadIdx.x == 0) scratch->partials[blockIdx.x] = p;
+}
+
+// The same for grids of many tiles, one partial per tile.
+template <bool LIN>
+__global__ void __launch_bounds__(256, 3) k_residual_tile64_noalloc(
+    int n, const double* __restrict__ phi, const double* __restrict__ delta, double a, double b,
+    const double* __restrict__ f, double* __restrict__ dout, OpConst64 c,
+    NoAllocScratch* __restrict__ scratch) {
+  __shared__ TileShared S;
+  Partial p;
+  partial_init(p);
+  tile_defects<LIN>(
+      n, phi, c, (int)blockIdx.x * kTileX, (int)blockIdx.y * kTileY, (int)blockIdx.z * kTileZ, S,
+      [&](int id) { return fma(a, delta[id], b); },
+      [&](int id, int, int, int, double d, double, bool g) {
+        if (f) d -= f[id];
+        if (dout) dout[id] = d;
+        partial_add(p, d, g);
+      });
+  p = tile_reduce(p, S);
+  if (threadIdx.x == 0) scratch->partials[tile_index()] = p;
 }
 
 // Device address of the scratch array, looked up once per device.  Host threads
@@ -130,8 +149,14 @@ extern "C" mg_status mg_op_residual_noalloc(int n, const double* phi, const doub
   const OpConst64 c = make_op64(n, alpha, kappa, branch);
   double a, b;
   src_coefficients(c, kappa, &a, &b);
-  const unsigned nb = (unsigned)((cells + kNoAllocThreads - 1) / kNoAllocThreads);
-  k_residual64_noalloc<<<nb, kNoAllocThreads, 0, s>>>(n, phi, delta, a, b, f, d, c, scratch);
+  const bool tiles = in_tiles(n, c);
+  const unsigned nb =
+      tiles ? tile_count(n) : (unsigned)((cells + kNoAllocThreads - 1) / kNoAllocThreads);
+  if (tiles)
+    (c.mode == OP_LINEAR ? k_residual_tile64_noalloc<true> : k_residual_tile64_noalloc<false>)
+        <<<tile_grid(n), 256, 0, s>>>(n, phi, delta, a, b, f, d, c, scratch);
+  else
+    k_residual64_noalloc<<<nb, kNoAllocThreads, 0, s>>>(n, phi, delta, a, b, f, d, c, scratch);
   count_launches(1);
   launch_finalize(s, scratch->partials, (int)nb, (double)cells, 1, &scratch->scalars);
   cudaError_t e = cudaGetLastError();

@@ -7,9 +7,9 @@
 // SM), finds the largest exponent, and converts each value once, to a unit 2^-59 of it.
 // Then no cell converts anything: 1.5 conversions per cell instead of 18 or 19.
 //
-// A value lost below the unit is less than an FP64 addition loses as long as the stencil
-// holds a value within 2^-6 of the tile's largest; tile_small finds the others, which take
-// their values from memory (cells at a zero of the field in a steep tile, about none).
+// What is cut off below the unit is less than FP64 additions lose as long as the stencil
+// holds a value within 2^-7 of the tile's largest; tile_small finds the others (cells at a
+// zero of the field in a steep tile), which take their values from memory.
 // Tiles without such a unit (infinities, NaN, extreme exponents) go cell by cell too.
 #pragma once
 
@@ -32,6 +32,27 @@ constexpr int kTileWords = kTilePlane * (kTileZ + 2);
 __host__ __device__ inline dim3 tile_grid(int n) {
   return dim3((unsigned)(n + kTileX - 1) / kTileX, (unsigned)(n + kTileY - 1) / kTileY,
               (unsigned)(n + kTileZ - 1) / kTileZ);
+}
+
+__host__ __device__ inline unsigned tile_count(int n) {
+  const dim3 g = tile_grid(n);
+  return g.x * g.y * g.z;
+}
+
+// Whether a level runs in tiles: its operator in the square-root or the linear form.  The
+// others (a splitting constant of its own, |alpha| < 1e-4) divide and would cost the tile
+// kernels the registers of a fourth CTA per SM; their cells go one by one.
+__host__ __device__ inline bool in_tiles(int n, const OpConst64& c) {
+  return n >= kTileMinSide && (c.mode == OP_SQRT || c.mode == OP_LINEAR);
+}
+// Its colour stages: with the plain step (omega = 1) only.
+__host__ __device__ inline bool smooth_in_tiles(int n, const OpConst64& c) {
+  return in_tiles(n, c) && c.omega == 1.0;
+}
+
+// The tile's place in the order of a launch over tile_grid.
+__device__ __forceinline__ unsigned tile_index() {
+  return blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
 }
 
 struct TileShared {
@@ -57,6 +78,29 @@ __device__ __forceinline__ float tile_max(float m, long long b) {
   float r;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(m), "f"(fabsf(__int_as_float(fix_hi(b)))));
   return r;
+}
+
+// The exponent field (in place) of the largest of all threads' values, -1 where the tile
+// has no unit; every thread gets the same.
+template <int NV>
+__device__ __forceinline__ int tile_exponent(const long long (&v)[NV], TileShared& S) {
+  float fm = 0.f;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) fm = tile_max(fm, v[k]);
+  int em = __reduce_max_sync(0xffffffffu, __float_as_int(fm) & 0x7fffffff);
+  if ((threadIdx.x & 31) == 0) S.em[threadIdx.x >> 5] = em;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) em = max(em, S.em[k]);
+  if (em < (kFixMinExp << 20) || em >= ((kFixMaxExp + 1) << 20)) {
+    long long any = em;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) any |= v[k] << 1;
+    // a tile of zeros has every unit
+    if (__syncthreads_or(any != 0)) return -1;
+    em = 1023 << 20;
+  }
+  return em & 0x7ff00000;
 }
 
 // Which values of a tile a thread (of 256) loads, and where they go.  For a stage of a
@@ -128,7 +172,7 @@ __device__ __forceinline__ TileMap tile_map(int n, int x0, int y0, int colour) {
 // 2^ue.  False (for every thread): it has none.
 __device__ __forceinline__ bool tile_load(int n, const double* __restrict__ phi, int z0,
                                           const TileMap& T, TileShared& S, int& ue) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int w = threadIdx.x >> 5;
   const int n2 = n * n;
   auto zoff = [&](int z) {
     const int k = z0 - 1 + z;
@@ -154,23 +198,8 @@ __device__ __forceinline__ bool tile_load(int n, const double* __restrict__ phi,
   v[16] = T.ze >= 0 ? rd(zoff(T.ze) + T.ge[1]) : 0;
   v[17] = rd(zoff(T.zl[0]) + T.gl[0]);
   v[18] = T.zl[1] >= 0 ? rd(zoff(T.zl[1]) + T.gl[1]) : 0;
-  float fm = 0.f;
-#pragma unroll
-  for (int k = 0; k < 19; ++k) fm = tile_max(fm, v[k]);
-  int em = __reduce_max_sync(0xffffffffu, __float_as_int(fm) & 0x7fffffff);
-  if (lane == 0) S.em[w] = em;
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 8; ++k) em = max(em, S.em[k]);
-  if (em < (kFixMinExp << 20) || em >= ((kFixMaxExp + 1) << 20)) {
-    long long any = em;
-#pragma unroll
-    for (int k = 0; k < 19; ++k) any |= v[k] << 1;
-    // a tile of zeros has every unit
-    if (__syncthreads_or(any != 0)) return false;
-    em = 1023 << 20;
-  }
-  em &= 0x7ff00000;
+  const int em = tile_exponent(v, S);
+  if (em < 0) return false;
   ue = (em >> 20) - 1082;
 #pragma unroll
   for (int z = 0; z < 10; ++z)
@@ -185,28 +214,15 @@ __device__ __forceinline__ bool tile_load(int n, const double* __restrict__ phi,
   return true;
 }
 
-// The forms of a cell where a value of theirs is small: face, M from N and sh of fix_quad.
-// In FP64 where no value around the cell (at place o of `row`, its x - 1 at l) reaches
-// 2^-7 of the unit's range, so that FP64 could resolve the stencil better.
-struct TileForms {
-  double face, M;
-};
-static __device__ __noinline__ TileForms tile_forms_small(long long face, unsigned long long N,
-                                                          int e, int ue, const long long* row,
-                                                          int o, int l, const double* at,
-                                                          NbrOff nbr) {
-  auto mag = [](long long v) { return (unsigned)(fix_hi(v) ^ (fix_hi(v) >> 31)); };
-  const unsigned top = mag(row[l]) | mag(row[l + 1]) | mag(row[o + kTileRow]) |
-                       mag(row[o - kTileRow]) | mag(row[o + kTilePlane]) |
-                       mag(row[o - kTilePlane]);
-  TileForms r;
-  if (top < (1u << 21)) {
-    stencil_forms_fp64(at, nbr, 18, &r.face, &r.M);
-  } else {
-    r.face = fix_signed(face, FixRef{0, ue, false});
-    r.M = fix_double(N, e);
-  }
-  return r;
+// Whether no value around the cell reaches 2^-7 of the tile's range (row[o]: its place,
+// row[l], row[r]: its neighbours in x), so that FP64 could resolve the stencil better.
+__device__ __forceinline__ unsigned tile_mag(long long v) {
+  return (unsigned)(fix_hi(v) ^ (fix_hi(v) >> 31));
+}
+__device__ __forceinline__ bool tile_small(const long long* row, int o, int l, int r) {
+  return (tile_mag(row[l]) | tile_mag(row[r]) | tile_mag(row[o + kTileRow]) |
+          tile_mag(row[o - kTileRow]) | tile_mag(row[o + kTilePlane]) |
+          tile_mag(row[o - kTilePlane])) < (1u << 21);
 }
 
 // A colour stage on the tile at (x0, y0, z0) (256 threads): four cells per thread, on
@@ -221,7 +237,9 @@ static __device__ __noinline__ TileForms tile_forms_small(long long face, unsign
 // 205 MB read and 40 MB written at 256^3 would take 36 us at the measured copy rate.
 // Tiles 16 planes deep, or several tiles per CTA one after the other, gained 1 % at 512^3
 // and lost at 256^3.
-template <bool F>
+// Cells that need another path (a value of theirs small against the tile, a vanishing or
+// infinite discriminant) are left for the end: no other cell of the stage reads them.
+template <bool F, bool LIN>
 __device__ __forceinline__ void b_smooth_tile64(int n, double* __restrict__ phi,
                                                 const double* __restrict__ src,
                                                 const double* __restrict__ f,
@@ -233,74 +251,349 @@ __device__ __forceinline__ void b_smooth_tile64(int n, double* __restrict__ phi,
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int p = w & 1, jj = (w >> 1) * 2 + (lane >> 4), m = lane & 15;
   const int px = (colour ^ p) & 1, py = ((colour >> 1) ^ p) & 1;
-  const int i = x0 + 2 * m + px, j = y0 + 2 * jj + py;
-  const int o = px ? 18 + m : m, l = px ? m : 17 + m;
+  const int i = x0 + 2 * m + px, j = y0 + 2 * jj + py, k0 = z0 + p;
   const int n2 = n * n;
   typedef unsigned long long u64;
   int ue;
   const bool ok = tile_load(n, phi, z0, T, S, ue);
   if (i >= n || j >= n) return;
   const double s_c = S.scalar;
-  int id = (z0 + p) * n2 + j * n + i;
-  if (!ok) {
-    for (int k = z0 + p; k < z0 + kTileZ && k < n; k += 2)
-      cell_smooth64_at(n, phi, src, f, s_c, c, i, j, k);
-    return;
-  }
-  const long long* row = S.v + (p + 1) * kTilePlane + (2 * jj + py + 1) * kTileRow;
-  auto at = [&](int q) { return (u64)row[q]; };
-  u64 cz = at(o - kTilePlane), dx = at(l + 1 - kTilePlane) - at(l - kTilePlane),
-      dy = at(o + kTileRow - kTilePlane) - at(o - kTileRow - kTilePlane);
+  unsigned rare = 0xf;
+  if (ok) {
+    rare = 0;
+    const int o = px ? 18 + m : m, l = px ? m : 17 + m;
+    const long long* row = S.v + (p + 1) * kTilePlane + (2 * jj + py + 1) * kTileRow;
+    auto at = [&](int q) { return (u64)row[q]; };
+    u64 cz = at(o - kTilePlane), dx = at(l + 1 - kTilePlane) - at(l - kTilePlane),
+        dy = at(o + kTileRow - kTilePlane) - at(o - kTileRow - kTilePlane);
+    int id = k0 * n2 + j * n + i;
 #pragma unroll 1
-  for (int k = z0 + p; k < z0 + kTileZ && k < n; k += 2, id += 2 * n2, row += 2 * kTilePlane) {
-    const double sv = src[id];
-    const double fv = F ? f[id] : 0.0;
-    const u64 sx = at(l) + at(l + 1), sy = at(o + kTileRow) + at(o - kTileRow);
-    const u64 cz1 = at(o + kTilePlane), dx1 = at(l + 1 + kTilePlane) - at(l + kTilePlane),
-              dy1 = at(o + kTileRow + kTilePlane) - at(o - kTileRow + kTilePlane);
-    const u64 sz = cz + cz1;
-    const long long face = (long long)(sx + sy + sz);
-    u64 N = 0;
-    int sh = 0;
-    unsigned tq = 1;
-    if (c.mode != OP_LINEAR) {
-      const long long a[3] = {(long long)(sx - sy), (long long)(sx - sz), (long long)(sy - sz)};
-      const long long cc[3] = {(long long)((at(l + 1 + kTileRow) + at(l - kTileRow)) -
-                                           (at(l + 1 - kTileRow) + at(l + kTileRow))),
-                               (long long)(dx1 - dx), (long long)(dy1 - dy)};
-      N = fix_quad(a, cc, sh, tq);
+    for (int s = 0; s < 4 && k0 + 2 * s < n; ++s, id += 2 * n2, row += 2 * kTilePlane) {
+      const double sv = src[id];
+      const double fv = F ? f[id] : 0.0;
+      const u64 sx = at(l) + at(l + 1), sy = at(o + kTileRow) + at(o - kTileRow);
+      const u64 cz1 = at(o + kTilePlane), dx1 = at(l + 1 + kTilePlane) - at(l + kTilePlane),
+                dy1 = at(o + kTileRow + kTilePlane) - at(o - kTileRow + kTilePlane);
+      const u64 sz = cz + cz1;
+      const long long face = (long long)(sx + sy + sz);
+      u64 N = 0;
+      int sh = 0;
+      unsigned tq = 1;
+      if (!LIN) {
+        const long long a[3] = {(long long)(sx - sy), (long long)(sx - sz), (long long)(sy - sz)};
+        const long long cc[3] = {(long long)((at(l + 1 + kTileRow) + at(l - kTileRow)) -
+                                             (at(l + 1 - kTileRow) + at(l + kTileRow))),
+                                 (long long)(dx1 - dx), (long long)(dy1 - dy)};
+        N = fix_quad(a, cc, sh, tq);
+      }
+      cz = cz1;
+      dx = dx1;
+      dy = dy1;
+      const unsigned fs = (unsigned)(fix_hi(face) >> 31);
+      const u64 fm = ((u64)face ^ fix_words(fs, fs)) - fix_words(fs, fs);
+      const unsigned ft = (unsigned)(fm >> 32);
+      bool bad = min(ft, tq) == 0 || ((ft | tq) < (1u << 24) && tile_small(row, o, l, l + 1));
+      double acc = F ? fma(fv, -c.h2_6, s_c) : s_c;
+      if (LIN) {
+        acc = fma(-c.h2_6, sv, acc);
+      } else {
+        const double q = fma(c.e1, fix_double_top(N, 64 - 2 * sh + 2 * ue), sv);
+        bad = bad || !fix_normal(q);
+        acc = fma(c.upd_s, sqrt_fix_normal(q), acc);
+      }
+      if (bad)
+        rare |= 1u << s;
+      else
+        phi[id] = fma(fix_double_top(fm, ue, fs & 0x80000000u), 1.0 / 6.0, acc);
     }
-    cz = cz1;
-    dx = dx1;
-    dy = dy1;
-    const int qe = 64 - 2 * sh + 2 * ue;
-    const unsigned fs = (unsigned)(fix_hi(face) >> 31);
-    const u64 fm = ((u64)face ^ fix_words(fs, fs)) - fix_words(fs, fs);
-    const unsigned ft = (unsigned)(fm >> 32);
-    double fd, M;
-    if (min(ft, tq) != 0 && (ft | tq) >= (1u << 24)) {
-      fd = fix_double_top(fm, ue, fs & 0x80000000u);
-      M = fix_double_top(N, qe);
-    } else {
-      const TileForms t = tile_forms_small(face, N, qe, ue, row, o, l, phi + id,
-                                           nbr_offsets(i, j, k, n));
-      fd = t.face;
-      M = t.M;
-    }
-    double acc = F ? fma(fv, -c.h2_6, s_c) : s_c;
-    if (c.mode == OP_SQRT) {
-      acc = fma(c.upd_s, sqrt_clamped_fix(fma(c.e1, M, sv)), acc);
-    } else {
-      double q;
-      bool g;
-      acc = fma(-c.h2_6, root_of_M(M, sv, c, q, g), acc);
-    }
-    const double v = fma(fd, 1.0 / 6.0, acc);
-    if (not_one(c.omega))
-      relax64(phi + id, v, c.omega);
-    else
-      phi[id] = v;
   }
+#pragma unroll 1
+  for (int s = 0; rare != 0; ++s, rare >>= 1) {
+    const int k = k0 + 2 * s;
+    if ((rare & 1) && k < n) cell_smooth64_at(n, phi, src, f, s_c, c, i, j, k);
+  }
+}
+
+// The whole tile, every row in the order of x (x0 - 1 first): for the kernels that visit
+// every cell.  Loads as tile_load: rows w and w + 8 of each plane, the last two rows of the
+// planes, then the ends of the rows.
+__device__ __forceinline__ bool tile_load_all(int n, const double* __restrict__ phi, int x0,
+                                              int y0, int z0, TileShared& S, int& ue) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int n2 = n * n;
+  auto wrap = [n](int v) { return v < 0 ? v + n : (v >= n ? v - n : v); };
+  auto gxy = [&](int x, int y) { return wrap(y0 - 1 + y) * n + wrap(x0 + x); };
+  auto zoff = [&](int z) { return wrap(z0 - 1 + z) * n2; };
+  auto rd = [&](int q) { return __double_as_longlong(phi[q]); };
+  long long v[25];
+  const int g0 = gxy(lane, w), g1 = gxy(lane, w + 8);
+  if (z0 > 0 && z0 + kTileZ < n) {
+    const double* p0 = phi + (z0 - 1) * n2 + g0;
+    const double* p1 = phi + (z0 - 1) * n2 + g1;
+#pragma unroll
+    for (int z = 0; z < 10; ++z) {
+      v[2 * z] = __double_as_longlong(p0[(long long)z * n2]);
+      v[2 * z + 1] = __double_as_longlong(p1[(long long)z * n2]);
+    }
+  } else {
+#pragma unroll
+    for (int z = 0; z < 10; ++z) {
+      v[2 * z] = rd(zoff(z) + g0);
+      v[2 * z + 1] = rd(zoff(z) + g1);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int e = w + 8 * r;
+    v[20 + r] = e < 20 ? rd(zoff(e >> 1) + gxy(lane, 16 + (e & 1))) : 0;
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int h = threadIdx.x + 256 * r, row = h >> 1, z = row / 18, y = row - 18 * z;
+    v[23 + r] = row < 180 ? rd(zoff(z) + gxy((h & 1) ? 32 : -1, y)) : 0;
+  }
+  const int em = tile_exponent(v, S);
+  if (em < 0) return false;
+  ue = (em >> 20) - 1082;
+  long long* t = S.v + w * kTileRow + lane + 1;
+#pragma unroll
+  for (int z = 0; z < 10; ++z) {
+    t[z * kTilePlane] = tile_convert(v[2 * z], em);
+    t[z * kTilePlane + 8 * kTileRow] = tile_convert(v[2 * z + 1], em);
+  }
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int e = w + 8 * r;
+    if (e < 20)
+      S.v[(e >> 1) * kTilePlane + (16 + (e & 1)) * kTileRow + lane + 1] =
+          tile_convert(v[20 + r], em);
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int h = threadIdx.x + 256 * r, row = h >> 1;
+    if (row < 180) S.v[row * kTileRow + ((h & 1) ? 33 : 0)] = tile_convert(v[23 + r], em);
+  }
+  __syncthreads();
+  return true;
+}
+
+// What a column of cells passes from plane to plane: value, differences across in x and y.
+struct TilePlane {
+  unsigned long long c, dx, dy;
+};
+__device__ __forceinline__ TilePlane tile_plane(const long long* q) {
+  typedef unsigned long long u64;
+  return TilePlane{(u64)q[0], (u64)q[1] - (u64)q[-1], (u64)q[kTileRow] - (u64)q[-kTileRow]};
+}
+
+// The defect L phi (without a right-hand side) of the cell at q in the tile (tile_load_all),
+// between the planes lo and up.  False: it needs another path, as in b_smooth_tile64.
+template <bool LIN>
+__device__ __forceinline__ bool tile_defect(const long long* q, const TilePlane& lo,
+                                            const TilePlane& mid, const TilePlane& up, int ue,
+                                            double src, const OpConst64& c, double& d, double& qd) {
+  typedef unsigned long long u64;
+  auto v = [&](int k) { return (u64)q[k]; };
+  const u64 sx = v(1) + v(-1), sy = v(kTileRow) + v(-kTileRow), sz = lo.c + up.c;
+  // half of the difference: twelve values would pass 64 bits
+  const long long lap = ((long long)(sx + sy + sz) >> 1) - 3 * (long long)mid.c;
+  u64 N = 0;
+  int sh = 0;
+  unsigned tq = 1;
+  if (!LIN) {
+    const long long a[3] = {(long long)(sx - sy), (long long)(sx - sz), (long long)(sy - sz)};
+    const long long cc[3] = {(long long)((v(kTileRow + 1) + v(-kTileRow - 1)) -
+                                         (v(-kTileRow + 1) + v(kTileRow - 1))),
+                             (long long)(up.dx - lo.dx), (long long)(up.dy - lo.dy)};
+    N = fix_quad(a, cc, sh, tq);
+  }
+  bool bad = tq == 0 || ((tile_mag((long long)mid.c) << 3 | tq) < (1u << 24) &&
+                         tile_small(q, 0, -1, 1));
+  double D = src;
+  qd = 1.0;
+  if (!LIN) {
+    qd = fma(c.e1, fix_double_top(N, 64 - 2 * sh + 2 * ue), src);
+    bad = bad || !fix_normal(qd);
+    D = fma(c.k2s, sqrt_fix_normal(qd), -c.k2);
+  }
+  d = fma(fix_signed(lap, FixRef{0, ue + 1, false}), c.inv_h2, -D);
+  return !bad;
+}
+
+// The defect kernels, 512^3: residual 13.1 -> 1.94 ms, residual with restriction 10.5 ->
+// 2.46 ms, hand-off to FP32 10.5 -> 3.38 ms (256^3 residual 1646 -> 253 us).  Per cell three
+// to five FP64 instructions remain (the FP64 pipe is about half busy), and three CTAs per SM
+// leave latency in sight; four, at 64 registers, spilled and took 3 % longer.
+//
+// Visit every cell of the tile at (x0, y0, z0): cell(id, i, j, k, defect, q, guard) with
+// src(id) its source term.  A thread takes two columns of eight cells, side by side in y,
+// the cells that need another path last.
+template <bool LIN, typename Src, typename Cell>
+__device__ __forceinline__ void tile_defects(int n, const double* __restrict__ phi,
+                                             const OpConst64& c, int x0, int y0, int z0,
+                                             TileShared& S, Src src, Cell cell) {
+  int ue;
+  const bool ok = tile_load_all(n, phi, x0, y0, z0, S, ue);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = x0 + lane, j0 = y0 + 2 * w, n2 = n * n;
+  if (i >= n || j0 >= n) return;  // n is even
+  unsigned rare = 0xffff;
+  if (ok) {
+    rare = 0;
+#pragma unroll 1
+    for (int y = 0; y < 2; ++y) {
+      const long long* q = S.v + kTilePlane + (2 * w + y + 1) * kTileRow + lane + 1;
+      TilePlane lo = tile_plane(q - kTilePlane), mid = tile_plane(q);
+      int id = z0 * n2 + (j0 + y) * n + i;
+#pragma unroll 1
+      for (int s = 0; s < kTileZ && z0 + s < n; ++s, id += n2, q += kTilePlane) {
+        const TilePlane up = tile_plane(q + kTilePlane);
+        double d, qd;
+        const bool good = tile_defect<LIN>(q, lo, mid, up, ue, src(id), c, d, qd);
+        lo = mid;
+        mid = up;
+        if (good)
+          cell(id, i, j0 + y, z0 + s, d, qd, false);
+        else
+          rare |= 1u << (8 * y + s);
+      }
+    }
+  }
+#pragma unroll 1
+  for (int s = 0; rare != 0; ++s, rare >>= 1) {
+    const int j = j0 + (s >> 3), k = z0 + (s & 7);
+    if (!(rare & 1) || k >= n) continue;
+    const int id = k * n2 + j * n + i;
+    double qd;
+    bool g;
+    const double d = cell_defect_fix64(phi, n, i, j, k, id, src(id), c, qd, g);
+    cell(id, i, j, k, d, qd, g);
+  }
+}
+
+// block_reduce of the 256 threads, in the tile's own memory.
+__device__ __forceinline__ Partial tile_reduce(Partial p, TileShared& S) {
+  Partial* sh = reinterpret_cast<Partial*>(S.v);
+  p = warp_reduce(p);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = p;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    Partial q;
+    partial_init(q);
+    if (threadIdx.x < 8) q = sh[threadIdx.x];
+    p = warp_reduce(q);
+  }
+  return p;
+}
+
+static __device__ __noinline__ double tile_defect_rare(const double* phi, int n, int i, int j,
+                                                       int k, double src, const OpConst64* c,
+                                                       bool* g) {
+  double q;
+  return cell_defect_fix64(phi, n, i, j, k, lidx(i, j, k, n), src, *c, q, *g);
+}
+
+// Residual restriction of a tile (b_residual_restrict64).  A thread takes a column of 2 x 1
+// fine cells in y and x, two planes at a time, and shares a coarse cell with its neighbour
+// lane in x.  R phi is the exact sum of the eight children, rounded once, where that is not
+// small against the tile.  Returns the tile's partial (thread 0).
+template <bool F, bool LIN>
+__device__ __forceinline__ Partial b_residual_restrict_tile64(
+    int nf, const double* __restrict__ phi, const double* __restrict__ src,
+    const double* __restrict__ f, const OpConst64& c, double* __restrict__ phi_c,
+    double* __restrict__ phihat_c, double* __restrict__ rd_c, int x0, int y0, int z0,
+    TileShared& S) {
+  int ue;
+  const bool ok = tile_load_all(nf, phi, x0, y0, z0, S, ue);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = x0 + lane, j0 = y0 + 2 * w, n2 = nf * nf, nc = nf >> 1;
+  const bool in = i < nf && j0 < nf;  // nf is even: whole coarse cells
+  Partial p;
+  partial_init(p);
+  double sum = 0.0;
+  long long kmax = order_key(-INFINITY), kmin = order_key(INFINITY);
+  const long long* q[2];
+  TilePlane lo[2], mid[2];
+#pragma unroll
+  for (int y = 0; y < 2; ++y) {
+    q[y] = S.v + kTilePlane + (2 * w + y + 1) * kTileRow + lane + 1;
+    lo[y] = tile_plane(q[y] - kTilePlane);
+    mid[y] = tile_plane(q[y]);
+  }
+#pragma unroll 1
+  for (int k0 = z0; k0 < z0 + kTileZ && k0 < nf; k0 += 2) {
+    double sd = 0.0;
+    unsigned long long sphi = 0;
+    if (in) {
+#pragma unroll
+      for (int ch = 0; ch < 4; ++ch) {
+        const int y = ch & 1, k = k0 + (ch >> 1), j = j0 + y;
+        const int id = k * n2 + j * nf + i;
+        double qd, d;
+        bool g = false, good = false;
+        if (ok) {
+          const TilePlane up = tile_plane(q[y] + kTilePlane);
+          good = tile_defect<LIN>(q[y], lo[y], mid[y], up, ue, src[id], c, d, qd);
+          sphi += mid[y].c;
+          lo[y] = mid[y];
+          mid[y] = up;
+          q[y] += kTilePlane;
+        }
+        if (!good) d = tile_defect_rare(phi, nf, i, j, k, src[id], &c, &g);
+        if (F) d -= f[id];
+        const bool fin = finite_bits(d);
+        const long long key = order_key(d);
+        kmax = (fin && key > kmax) ? key : kmax;
+        kmin = (fin && key < kmin) ? key : kmin;
+        p.nonfinite += fin ? 0 : 1;
+        p.guards += g ? 1 : 0;
+        sd += d;
+      }
+    }
+    // with a non-finite defect the level has no residual, and its sum no use
+    if (p.nonfinite == 0) sum += sd;
+    const double sd2 = sd + __shfl_xor_sync(0xffffffffu, sd, 1);
+    const unsigned long long sp2 = sphi + __shfl_xor_sync(0xffffffffu, sphi, 1);
+    if (in && (lane & 1) == 0) {
+      const int cid = (k0 >> 1) * nc * nc + (j0 >> 1) * nc + (i >> 1);
+      const int h = (int)(sp2 >> 32);
+      double r;
+      if (ok && (unsigned)(h ^ (h >> 31)) >= (1u << 24)) {
+        r = fix_signed((long long)sp2, FixRef{0, ue - 3, false});
+      } else {
+        r = 0.0;
+#pragma unroll 1
+        for (int ch = 0; ch < 8; ++ch)
+          r += phi[(k0 + (ch >> 2)) * n2 + (j0 + ((ch >> 1) & 1)) * nf + i + (ch & 1)];
+        r *= 0.125;
+      }
+      phi_c[cid] = r;
+      phihat_c[cid] = r;
+      rd_c[cid] = sd2 * 0.125;
+    }
+  }
+  p.sum = sum;
+  if (kmax >= kmin) {
+    p.dmax = from_order_key(kmax);
+    p.dmin = from_order_key(kmin);
+  }
+  return tile_reduce(p, S);
+}
+
+// The FAS right-hand side of a tile (cell_fas_rhs64).
+template <bool LIN>
+__device__ __forceinline__ void b_fas_rhs_tile64(int nc, const double* __restrict__ phi_c,
+                                                 const double* __restrict__ src_c,
+                                                 double* __restrict__ f_c, const OpConst64& c,
+                                                 const LevelScalars* __restrict__ fine_sc,
+                                                 LevelScalars* __restrict__ coarse_sc, int x0,
+                                                 int y0, int z0, TileShared& S) {
+  if ((x0 | y0 | z0) == 0 && threadIdx.x == 0) coarse_sc->lambda = 0.0;
+  const double lam = fine_sc->lambda;
+  tile_defects<LIN>(
+      nc, phi_c, c, x0, y0, z0, S, [&](int id) { return src_c[id]; },
+      [&](int id, int, int, int, double L, double, bool) { f_c[id] = L - f_c[id] + lam; });
 }
 
 }  // namespace mg

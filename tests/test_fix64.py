@@ -89,10 +89,13 @@ def stencil(kind, rng):
         return base * noise * (rng.random(19) < 0.5)
     if kind == "far":  # one large value, the others down to 2^-80 of it
         return base * noise * 2.0 ** -rng.integers(0, 80, 19)
+    if kind == "checker":  # the largest sums: faces against the centre
+        return base * (2 - 2.0 ** -52) * np.where(np.arange(19) < 6, 1.0, -1.0)
     return base * np.where(rng.random(19) < 0.5, 1.0, 1 - 2.0 ** -53)  # "ulp"
 
 
-@pytest.mark.parametrize("kind", ["smooth", "flat", "edge", "signs", "rough", "zeros", "far", "ulp"])
+@pytest.mark.parametrize("kind", ["smooth", "flat", "edge", "signs", "rough", "zeros", "far", "ulp",
+                                  "checker"])
 def test_forms(lib, kind):
     rng = np.random.default_rng(5)
     for _ in range(400):

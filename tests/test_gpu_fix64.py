@@ -55,7 +55,7 @@ def field(kind, n, rng):
             "tiny": 1e-150 * noise}[kind]
 
 
-@pytest.mark.parametrize("n", [30, 66, 110, 112, 114, 134])
+@pytest.mark.parametrize("n", [30, 112, 114])
 @pytest.mark.parametrize("kind", ["one binade", "waves", "noise", "zero", "spikes", "tiny"])
 def test_sweep(n, kind):
     rng = np.random.default_rng(n)
