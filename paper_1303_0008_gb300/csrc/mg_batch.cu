@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) kb_residual_restrict64(const BItem* __res
 // coarse cells); mode 1: partials of a per-cell kernel (one per 256 cells).
 // use32: reduce into the FP32 inner scalars.  Level-0 scalars are copied to
 // it.out, and with clear_mu the inner compatibility constant is reset.
-__global__ void __launch_bounds__(256) kb_finalize(const BItem* __restrict__ items, int mode,
+__global__ void __launch_bounds__(1024) kb_finalize(const BItem* __restrict__ items, int mode,
                                                    int use32, int clear_mu) {
   const BItem& it = items[blockIdx.x];
   const long long cells = (long long)it.n * it.n * it.n;
@@ -466,7 +466,7 @@ struct BatchCycle {
   void finalize(int l, ListType src_type, int mode, int use32, int clear_mu) const {
     const StageList& one = L(l, T_ONE, src_type == T_RR ? P_DESC : P_HAS);
     if (one.count == 0) return;
-    kb_finalize<<<one.count, 256, 0, st>>>(one.d, mode, use32, clear_mu);
+    kb_finalize<<<one.count, 1024, 0, st>>>(one.d, mode, use32, clear_mu);
     count_launches(1);
   }
 

@@ -383,8 +383,8 @@ __device__ __forceinline__ void partial_add(Partial& p, double d, bool guard) {
 
 __device__ __forceinline__ void partial_merge(Partial& a, const Partial& b) {
   a.sum += b.sum;
-  a.dmax = fmax(a.dmax, b.dmax);
-  a.dmin = fmin(a.dmin, b.dmin);
+  if (order_key(b.dmax) > order_key(a.dmax)) a.dmax = b.dmax;
+  if (order_key(b.dmin) < order_key(a.dmin)) a.dmin = b.dmin;
   a.guards += b.guards;
   a.nonfinite += b.nonfinite;
 }

@@ -151,25 +151,98 @@ __global__ void __launch_bounds__(256) k_restrict_defects64(
   b_restrict_defects64(nf, phi, din, gin, phi_c, phihat_c, rd_c, partials, blockIdx.x);
 }
 
-// The coarse correction phihat_c <- phi_c - phihat_c (R phi is not needed after
-// the prolongation), then the prolongation from it: the subtraction is done once
-// per coarse cell instead of once per fine cell that reads it.
-__global__ void __launch_bounds__(256) k_correction64(long long cells,
-                                                      const double* __restrict__ phi_c,
-                                                      double* __restrict__ phihat_c) {
+// The prolongation of a large level by columns: a thread takes KZ coarse cells above one
+// another and their 8 KZ children, the CTA 32 x 8 columns.  A coarse plane's corrections
+// are formed once in shared memory, interpolated along x and y once (10 multiply-adds per
+// coarse cell) and used for the planes of children above and below: 3.7 FP64 instructions
+// per fine cell instead of 11 (19 with the corrections formed by each of their readers).
+// At 300^3 the kernel takes 223 instead of 873 us; in the FP64 solve of 512^3
+// the finest one 1.0 instead of 2.4 ms.  The FP64 pipe still bounds it.
+template <int KZ>
+__global__ void __launch_bounds__(256) k_prolong_column64(int nc, const double* __restrict__ phi_c,
+                                                          const double* __restrict__ phihat_c,
+                                                          double* __restrict__ phi_f) {
   PdlScope pdl_scope;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < cells) phihat_c[t] = phi_c[t] - phihat_c[t];
-}
-
-__global__ void __launch_bounds__(256) k_prolong_corr64(int nc, const double* __restrict__ corr_c,
-                                                        double* __restrict__ phi_f) {
-  PdlScope pdl_scope;
-  cell_prolong_corr64(nc, corr_c, phi_f, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+  constexpr int W = 34, H = 10;
+  __shared__ double e[2][W * H];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int I0 = (int)blockIdx.x * 32, J0 = (int)blockIdx.y * 8, K0 = (int)blockIdx.z * KZ;
+  auto wrap = [nc](int v) { return v < 0 ? v + nc : (v >= nc ? v - nc : v); };
+  int at[2];  // this thread's cells of a plane of the CTA's tile
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int q = threadIdx.x + 256 * r, y = q / W;
+    at[r] = wrap(J0 - 1 + y) * nc + wrap(I0 - 1 + q - W * y);
+  }
+  auto load = [&](int K, double* t) {
+    const long long p = (long long)wrap(K) * nc * nc;
+    t[threadIdx.x] = phi_c[p + at[0]] - phihat_c[p + at[0]];
+    if (threadIdx.x < W * H - 256)
+      t[threadIdx.x + 256] = phi_c[p + at[1]] - phihat_c[p + at[1]];
+  };
+  // (y side, x side) of the column's cell in a plane: towards -y or +y, -x or +x
+  auto interpolate = [&](const double* t, double (&b)[4]) {
+    double a[3][2];
+#pragma unroll
+    for (int y = 0; y < 3; ++y) {
+      const double* r = t + (w + y) * W + lane + 1;
+      a[y][0] = fma(3.0, r[0], r[-1]);
+      a[y][1] = fma(3.0, r[0], r[1]);
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      b[x] = fma(3.0, a[1][x], a[0][x]);
+      b[2 + x] = fma(3.0, a[1][x], a[2][x]);
+    }
+  };
+  double lo[4], mid[4], up[4];
+  load(K0 - 1, e[0]);
+  load(K0, e[1]);
+  __syncthreads();
+  interpolate(e[0], lo);
+  interpolate(e[1], mid);
+  __syncthreads();
+  const int I = I0 + lane, J = J0 + w, nf = 2 * nc;
+  const bool in = I < nc && J < nc;
+#pragma unroll 1
+  for (int s = 0; s < KZ && K0 + s < nc; ++s) {
+    const int K = K0 + s;
+    double* t = e[s & 1];
+    load(K + 1, t);
+    double2 v[4];
+    double2* f = reinterpret_cast<double2*>(phi_f + lidx(2 * I, 2 * J, 2 * K, nf));
+    const long long row = nf / 2, plane = (long long)nf * nf / 2;  // in pairs
+    if (in) {
+      v[0] = f[0];
+      v[1] = f[row];
+      v[2] = f[plane];
+      v[3] = f[plane + row];
+    }
+    __syncthreads();
+    interpolate(t, up);
+    if (in) {
+#pragma unroll
+      for (int y = 0; y < 2; ++y) {
+        v[y].x = fma(fma(3.0, mid[2 * y], lo[2 * y]), 1.0 / 64.0, v[y].x);
+        v[y].y = fma(fma(3.0, mid[2 * y + 1], lo[2 * y + 1]), 1.0 / 64.0, v[y].y);
+        v[2 + y].x = fma(fma(3.0, mid[2 * y], up[2 * y]), 1.0 / 64.0, v[2 + y].x);
+        v[2 + y].y = fma(fma(3.0, mid[2 * y + 1], up[2 * y + 1]), 1.0 / 64.0, v[2 + y].y);
+      }
+      f[0] = v[0];
+      f[row] = v[1];
+      f[plane] = v[2];
+      f[plane + row] = v[3];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      lo[q] = mid[q];
+      mid[q] = up[q];
+    }
+  }
 }
 
 // One block: reduce the partials in a fixed order and publish the scalars.
-__global__ void __launch_bounds__(256) k_finalize(const Partial* __restrict__ partials, int nparts,
+__global__ void __launch_bounds__(1024) k_finalize(const Partial* __restrict__ partials, int nparts,
                                                   double cells, int periodic,
                                                   LevelScalars* __restrict__ sc) {
   PdlScope pdl_scope;
@@ -263,20 +336,34 @@ __global__ void __launch_bounds__(256) k_sub_mean(long long cells, double* __res
   b_sub_mean(cells, x, sc, blockIdx.x);
 }
 
-// g = -(1/2) grad phi, central differences; out is 3 x n^3 (x, y, z).
-__global__ void __launch_bounds__(256) k_force64(int n, const double* __restrict__ phi,
+// x -2^k by the exponent, on the integer pipe (its FP64 product where that is not a normal
+// number).
+static __device__ __noinline__ double scale_rare(double x, int k) { return -scalbn(x, k); }
+__device__ __forceinline__ double neg_scale(double x, int k) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e == 0 || e + k < 1 || e + k > 2046) return scale_rare(x, k);
+  return __hiloint2double((hi + (k << 20)) ^ 0x80000000, __double2loint(x));
+}
+
+// g = -(1/2) grad phi, central differences; out is 3 x n^3 (x, y, z).  The factor
+// -(1/2) / (2h) = -n/4; log2n: of a power of two n, else -1.  512^3: 2060 -> 791 us with
+// the three products taken off the FP64 pipe, which bounded it; the three differences and
+// the 4.3 GB moved now take about the same.
+__global__ void __launch_bounds__(256) k_force64(int n, int log2n, const double* __restrict__ phi,
                                                  double* __restrict__ out) {
   PdlScope pdl_scope;
   const long long cells = (long long)n * n * n;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= cells) return;
-  const int i = (int)(t % n);
-  const int j = (int)((t / n) % n);
-  const int k = (int)(t / ((long long)n * n));
-  const double sc = -0.25 * (double)n;  // -(1/2) / (2h)
-  out[t] = sc * (phi[lidx(wrap_up(i, n), j, k, n)] - phi[lidx(wrap_dn(i, n), j, k, n)]);
-  out[cells + t] = sc * (phi[lidx(i, wrap_up(j, n), k, n)] - phi[lidx(i, wrap_dn(j, n), k, n)]);
-  out[2 * cells + t] = sc * (phi[lidx(i, j, wrap_up(k, n), n)] - phi[lidx(i, j, wrap_dn(k, n), n)]);
+  int i, j, k;
+  split3((unsigned)t, n, i, j, k);
+  const NbrOff o = nbr_offsets(i, j, k, n);
+  const double* c = phi + t;
+  const double d[3] = {c[o.xp] - c[o.xm], c[o.yp] - c[o.ym], c[o.zp] - c[o.zm]};
+  const double sc = -0.25 * (double)n;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    out[a * cells + t] = log2n >= 0 ? neg_scale(d[a], log2n - 2) : sc * d[a];
 }
 
 // ---------------------------------------------------------------------------
@@ -350,6 +437,14 @@ int tpb_for(long long items) {
   return (long long)blocks_for(items, 256) < 2LL * sms ? 64 : 256;
 }
 
+// 1024 threads (as the batch's) where there are partials for them; the order of the sums is
+// the same with fewer.
+void launch_finalize(cudaStream_t st, const Partial* partials, int nparts, double cells,
+                     int periodic, LevelScalars* sc) {
+  launch_k(k_finalize, 1, nparts > 256 ? 1024 : 256, 0, st, partials, nparts, cells, periodic, sc);
+  count_launches(1);
+}
+
 void launch_smooth64(cudaStream_t st, int n, double* phi, const double* src, const double* f,
                      const LevelScalars* sc, const OpConst64& c, int sweeps, EventPairs* timer) {
   const int hn = n / 2;
@@ -386,8 +481,8 @@ void launch_residual64(cudaStream_t st, int n, const double* phi, const double* 
     launch_k(c.mode == OP_LINEAR ? k_residual_tile64<true> : k_residual_tile64<false>, tile_grid(n), 256, 0, st, n, phi, src, f, dout, c, partials);
   else
     launch_k(k_residual64, nb, 256, 0, st, n, phi, src, f, dout, c, partials);
-  launch_k(k_finalize, 1, 256, 0, st, partials, (int)nb, (double)cells, periodic, sc);
-  count_launches(2);
+  launch_finalize(st, partials, (int)nb, (double)cells, periodic, sc);
+  count_launches(1);
 }
 
 void launch_residual_restrict64(cudaStream_t st, int nf, const double* phi, const double* src,
@@ -415,8 +510,8 @@ void launch_residual_restrict64(cudaStream_t st, int nf, const double* phi, cons
     launch_k(k_residual_restrict64, nb, 256, 0, st, nf, phi, src, f, c, phi_c, phihat_c, rd_c,
              partials);
   }
-  launch_k(k_finalize, 1, 256, 0, st, partials, (int)nb, (double)fcells, 1, sc);
-  count_launches(2);
+  launch_finalize(st, partials, (int)nb, (double)fcells, 1, sc);
+  count_launches(1);
 }
 
 void launch_fas_rhs64(cudaStream_t st, int nc, const double* phi_c, const double* src_c,
@@ -433,19 +528,24 @@ void launch_fas_rhs64(cudaStream_t st, int nc, const double* phi_c, const double
   count_launches(1);
 }
 
+// By columns from nc = 48 on (fine side 96, where CTAs of four cells deep columns reach
+// most SMs); deeper columns once they leave four CTAs per SM.  The columns' loads of pairs
+// need a 16-byte aligned field.
 void launch_prolong_correct64(cudaStream_t st, int nc, const double* phi_c,
-                              const double* phihat_c, double* phi_f, bool clobber_hat) {
+                              const double* phihat_c, double* phi_f) {
   const long long cells = 8LL * nc * nc * nc;
-  if (clobber_hat && cells >= kCorrectionMinFine) {
-    const long long cc = cells / 8;
-    double* corr = const_cast<double*>(phihat_c);
-    launch_k(k_correction64, blocks_for(cc, 256), 256, 0, st, cc, phi_c, corr);
-    launch_k(k_prolong_corr64, blocks_for(cells, 256), 256, 0, st, nc, (const double*)corr, phi_f);
-    count_launches(1);
-    return;
+  const unsigned bx = blocks_for(nc, 32), by = blocks_for(nc, 8);
+  if (nc >= 48 && reinterpret_cast<uintptr_t>(phi_f) % 16 == 0) {
+    if ((long long)bx * by * blocks_for(nc, 8) >= 608)
+      launch_k(k_prolong_column64<8>, dim3(bx, by, blocks_for(nc, 8)), 256, 0, st, nc, phi_c,
+               phihat_c, phi_f);
+    else
+      launch_k(k_prolong_column64<4>, dim3(bx, by, blocks_for(nc, 4)), 256, 0, st, nc, phi_c,
+               phihat_c, phi_f);
+  } else {
+    const int tpb = tpb_for(cells);
+    launch_k(k_prolong_correct64, blocks_for(cells, tpb), tpb, 0, st, nc, phi_c, phihat_c, phi_f);
   }
-  const int tpb = tpb_for(cells);
-  launch_k(k_prolong_correct64, blocks_for(cells, tpb), tpb, 0, st, nc, phi_c, phihat_c, phi_f);
   count_launches(1);
 }
 
@@ -476,20 +576,20 @@ void launch_affine64(cudaStream_t st, long long cells, const double* x, double* 
 
 void launch_gauge64(cudaStream_t st, long long cells, double* x, Partial* partials,
                     LevelScalars* sc) {
-  const unsigned nb = blocks_for(cells, 256);
+  const unsigned nb = blocks_for(cells, 256 * kSumCells);
   launch_k(k_sum_partials, nb, 256, 0, st, cells, x, partials);
-  launch_k(k_finalize, 1, 256, 0, st, partials, (int)nb, (double)cells, 1, sc);
-  launch_k(k_sub_mean, nb, 256, 0, st, cells, x, sc);
-  count_launches(3);
+  launch_finalize(st, partials, (int)nb, (double)cells, 1, sc);
+  launch_k(k_sub_mean, blocks_for(cells, 256), 256, 0, st, cells, x, sc);
+  count_launches(2);
 }
 
 // max |x - mean x| into sc->res (sc->lambda = mean x)
 void launch_spread64(cudaStream_t st, long long cells, const double* x, Partial* partials,
                      LevelScalars* sc) {
-  const unsigned nb = blocks_for(cells, 256);
+  const unsigned nb = blocks_for(cells, 256 * kSumCells);
   launch_k(k_sum_partials, nb, 256, 0, st, cells, x, partials);
-  launch_k(k_finalize, 1, 256, 0, st, partials, (int)nb, (double)cells, 1, sc);
-  count_launches(2);
+  launch_finalize(st, partials, (int)nb, (double)cells, 1, sc);
+  count_launches(1);
 }
 
 // out = x + a y
@@ -510,16 +610,11 @@ void launch_axpy64(cudaStream_t st, long long cells, const double* x, const doub
 
 void launch_force64(cudaStream_t st, int n, const double* phi, double* out) {
   const long long cells = (long long)n * n * n;
-  launch_k(k_force64, blocks_for(cells, 256), 256, 0, st, n, phi, out);
+  int log2n = -1;
+  if ((n & (n - 1)) == 0)
+    for (log2n = 0; (1 << log2n) < n;) ++log2n;
+  launch_k(k_force64, blocks_for(cells, 256), 256, 0, st, n, log2n, phi, out);
   count_launches(1);
 }
 
-}  // namespace mg
-
-namespace mg {
-void launch_finalize(cudaStream_t st, const Partial* partials, int nparts, double cells,
-                     int periodic, LevelScalars* sc) {
-  launch_k(k_finalize, 1, 256, 0, st, partials, nparts, cells, periodic, sc);
-  count_launches(1);
-}
 }  // namespace mg

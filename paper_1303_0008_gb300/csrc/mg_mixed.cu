@@ -244,7 +244,10 @@ __global__ void __launch_bounds__(256) k_prolong_correct32(int nc, const float* 
 }
 
 // ehat_c <- e_c - ehat_c (R e is not needed after the prolongation), then the
-// prolongation from it (as k_correction64 and k_prolong_corr64).
+// prolongation from it: the subtraction once per coarse cell instead of once per fine
+// cell that reads it, on levels from kCorrectionMinFine fine cells on.
+constexpr long long kCorrectionMinFine = 128LL * 128 * 128;
+
 __global__ void __launch_bounds__(256) k_correction32(long long cells, const float* __restrict__ e_c,
                                                       float* __restrict__ ehat_c) {
   PdlScope pdl_scope;
