@@ -215,7 +215,23 @@ __global__ void __launch_bounds__(256) kb_smooth32(const BItem* __restrict__ ite
                                                    int colour) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
-  b_smooth_colour32(it.n, it.e, it.phi0, it.q0, it.rhs, it.sc32, it.op32, colour, blk);
+  if (it.n < kColour32TileMin) {
+    b_smooth_colour32(it.n, it.e, it.phi0, it.q0, it.rhs, it.sc32, it.op32, colour, blk);
+    return;
+  }
+  __shared__ float s_mu;
+  if (threadIdx.x == 0) s_mu = (float)it.sc32->lambda;
+  __syncthreads();
+  const bool narrow = colour32_narrow(it.n);
+  const dim3 g = narrow ? colour32_grid<16>(it.n) : colour32_grid<32>(it.n);
+  const unsigned b = (unsigned)blk, r = b / g.x;
+  const int bx = (int)(b - r * g.x), by = (int)(r % g.y), bz = (int)(r / g.y);
+  if (narrow)
+    b_colour32_tile<16, false>(it.n, it.e, it.phi0, it.q0, it.rhs, s_mu, it.op32, colour, bx, by,
+                               bz);
+  else
+    b_colour32_tile<32, false>(it.n, it.e, it.phi0, it.q0, it.rhs, s_mu, it.op32, colour, bx, by,
+                               bz);
 }
 
 __global__ void __launch_bounds__(256) kb_residual_restrict32(const BItem* __restrict__ items,
@@ -261,7 +277,11 @@ static long long blocks_of(ListType t, const BItem& it) {
     case T_SM64:
       if (smooth_in_tiles(n, it.op)) return tile_count(n);
       return (cells / 4 + 255) / 256;
-    case T_SMOOTH: return (cells / 4 + 255) / 256;
+    case T_SMOOTH: {
+      if (n < kColour32TileMin) return (cells / 4 + 255) / 256;
+      const dim3 g = colour32_narrow(n) ? colour32_grid<16>(n) : colour32_grid<32>(n);
+      return (long long)g.x * g.y * g.z;
+    }
     case T_RR64:
       if (in_tiles(n, it.op)) return tile_count(n);
       return (cells / 8 + 255) / 256;

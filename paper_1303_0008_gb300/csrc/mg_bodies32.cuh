@@ -420,6 +420,97 @@ __device__ __forceinline__ void cell_smooth32_n_z2(float* __restrict__ e,
   e[idb] = gs_value32(seb, ddb, gb, mu, c);
 }
 
+// Face sums and cross differences around the cell at c0, of x parity P, from 8-byte pairs
+// as gather_n2, for any even side: o the neighbour offsets, `far` that of the pair beyond
+// the cell's own (x - 2 or x + 1, the wrap folded in).  The sums are gather_at's.
+template <int P>
+struct PairRows {
+  int far;
+  __device__ __forceinline__ void row(const float* r, float& vm, float& v0, float& vp) const {
+    if (P == 0) {
+      const float2 a = ld2(r + far), b = ld2(r);
+      vm = a.y;
+      v0 = b.x;
+      vp = b.y;
+    } else {
+      const float2 a = ld2(r - 1), b = ld2(r + far);
+      vm = a.x;
+      v0 = a.y;
+      vp = b.x;
+    }
+  }
+};
+
+template <int P>
+__device__ __forceinline__ StencilT<float> gather_pairs(const float* c0, const NbrOff& o, int far) {
+  const PairRows<P> R{far};
+  float cm, cc, cp, am, a0, ap, bm, b0, bp, fm, f0, fp, gm, g0, gp;
+  R.row(c0, cm, cc, cp);
+  R.row(c0 + o.yp, am, a0, ap);
+  R.row(c0 + o.ym, bm, b0, bp);
+  R.row(c0 + o.zp, fm, f0, fp);
+  R.row(c0 + o.zm, gm, g0, gp);
+  StencilT<float> s;
+  s.sx = cp + cm;
+  s.sy = a0 + b0;
+  s.sz = f0 + g0;
+  s.cxy = (ap + bm) - (bp + am);
+  s.cxz = (fp + gm) - (gp + fm);
+  s.cyz = (c0[o.yp + o.zp] + c0[o.ym + o.zm]) - (c0[o.yp + o.zm] + c0[o.ym + o.zp]);
+  return s;
+}
+
+// The colour stage of a side that is no power of two (or of many grids at once) in CTA
+// tiles: LX cells in x per warp (and 32 / LX rows), two warps in y by four in z.  CO as in
+// cell_smooth32_n.  The bits are cell_smooth32's.
+//
+// Pairs and tiles are what the power-of-two kernels gained from; here the offsets are
+// known at run time only: all stages of a 448^3 solve 497 -> 424 ms, of a 192^3 solve 8.9 ->
+// 7.3 ms.  Two cells per thread on planes two apart, which pays there
+// from 256 on, lost 20 % (448^3: 310 us).
+template <int LX>
+__host__ __device__ inline dim3 colour32_grid(int n) {
+  const int hn = n / 2, rows = 2 * (32 / LX);
+  return dim3((unsigned)(hn + LX - 1) / LX, (unsigned)(hn + rows - 1) / rows,
+              (unsigned)(n + 3) / 4);
+}
+template <int LX, bool CO>
+__device__ __forceinline__ void b_colour32_tile(int n, float* __restrict__ e,
+                                                const float* __restrict__ phi0,
+                                                const float* __restrict__ q0,
+                                                const float* __restrict__ g, float mu,
+                                                const OpConst32& c, int colour, int bx, int by,
+                                                int bz) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, hn = n >> 1;
+  const int m = bx * LX + (lane & (LX - 1));
+  const int jj = (by * 2 + (w & 1)) * (32 / LX) + lane / LX;
+  const int k = bz * 4 + (w >> 1);
+  if (m >= hn || jj >= hn || k >= n) return;
+  const int par = (colour ^ k) & 1;
+  const int i = 2 * m + par, j = 2 * jj + (((colour >> 1) ^ k) & 1);
+  const int id = i + n * (j + n * k), t = (k * hn + jj) * hn + m;
+  const NbrOff o = nbr_offsets(i, j, k, n);
+  const int far = par ? o.xp : (i == 0 ? n - 2 : -2);
+  const float qv = CO ? q0[t] : q0[id], gv = CO ? g[t] : g[id];
+  StencilT<float> se, sp;
+  if (par) {
+    se = gather_pairs<1>(e + id, o, far);
+    if (!c.linear) sp = gather_pairs<1>(phi0 + id, o, far);
+  } else {
+    se = gather_pairs<0>(e + id, o, far);
+    if (!c.linear) sp = gather_pairs<0>(phi0 + id, o, far);
+  }
+  e[id] = gs_value32(se, c.linear ? 0.f : dD32(se, sp, qv, c), gv, mu, c);
+}
+
+// Sides that run so, and whether in warps of 16 cells in x: where they leave fewer lanes
+// idle.
+constexpr int kColour32TileMin = 32;
+__host__ __device__ inline bool colour32_narrow(int n) {
+  const int hn = n / 2;
+  return (hn + 15) / 16 * 16 < (hn + 31) / 32 * 32;
+}
+
 __device__ __forceinline__ void b_smooth_colour32(int n, float* __restrict__ e,
                                                          const float* __restrict__ phi0,
                                                          const float* __restrict__ q0,
@@ -526,6 +617,8 @@ __device__ __forceinline__ float fine_defect32(int nf, const float* __restrict__
   return fmaf(lap, c.inv_h2, -dd) - g[id];
 }
 
+// Measured and not kept here: the block of 4 x 4 x 4 values loaded once per coarse cell (128
+// registers; 448^3: 1014 to 1072 us against 855), the children's stencils from pairs (1262 us).
 __device__ __forceinline__ void b_residual_restrict32(
     int nf, const float* __restrict__ e, const float* __restrict__ phi0,
     const float* __restrict__ q0, const float* __restrict__ g, OpConst32 c,

@@ -100,6 +100,35 @@ __global__ void __launch_bounds__(256) k_smooth_colour32(int n, float* __restric
   b_smooth_colour32(n, e, phi0, q0, g, sc, c, colour, blockIdx.x);
 }
 
+// The colour stage of a side that is no power of two, in tiles (b_colour32_tile).
+template <int LX, bool CO>
+__global__ void __launch_bounds__(256) k_smooth_colour32_tile(int n, float* __restrict__ e,
+                                                              const float* __restrict__ phi0,
+                                                              const float* __restrict__ q0,
+                                                              const float* __restrict__ g,
+                                                              const LevelScalars* __restrict__ sc,
+                                                              OpConst32 c, int colour) {
+  PdlScope pdl_scope;
+  __shared__ float s_mu;
+  if (threadIdx.x == 0) s_mu = (float)sc->lambda;
+  __syncthreads();
+  b_colour32_tile<LX, CO>(n, e, phi0, q0, g, s_mu, c, colour, (int)blockIdx.x,
+                              (int)blockIdx.y, (int)blockIdx.z);
+}
+
+template <int LX>
+static void launch_colour32_tile(cudaStream_t st, int n, bool co, float* e, const float* phi0,
+                                 const float* q0, const float* g, const LevelScalars* sc,
+                                 const OpConst32& c, int colour) {
+  const dim3 grid = colour32_grid<LX>(n);
+  if (co)
+    launch_k(k_smooth_colour32_tile<LX, true>, grid, 256, 0, st, n, e, phi0, q0, g, sc, c,
+             colour);
+  else
+    launch_k(k_smooth_colour32_tile<LX, false>, grid, 256, 0, st, n, e, phi0, q0, g, sc, c,
+             colour);
+}
+
 constexpr int ilog2(unsigned v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }
 
 // Which of a colour's N^3/4 cells thread tid of a 256-thread CTA blk updates.
@@ -333,7 +362,7 @@ static mg_status mixed_prepare(Domain* d) {
     ok = ok && cudaMalloc(&L.rhs, b) == cudaSuccess;
     if (l > 0) ok = ok && cudaMalloc(&L.ehat, b) == cudaSuccess;
     if (sweep32_eligible(L.n)) ok = ok && cudaMalloc(&L.e2, b) == cudaSuccess;
-    if (l == 0 && L.n >= 64 && L.n <= 1024 && (L.n & (L.n - 1)) == 0) {
+    if (l == 0 && L.n >= 64) {
       ok = ok && cudaMalloc(&L.q0c, b) == cudaSuccess;
       ok = ok && cudaMalloc(&L.rhsc, b) == cudaSuccess;
     }
@@ -440,9 +469,18 @@ struct CycleMixed {
           case 256: stage(launch_colour32_n<256, true>, launch_colour32_n<256, false>); break;
           case 512: stage(launch_colour32_n<512, true>, launch_colour32_n<512, false>); break;
           case 1024: stage(launch_colour32_n<1024, true>, launch_colour32_n<1024, false>); break;
-          default:
-            launch_k(k_smooth_colour32, nb, 256, 0, st, L.n, L.e, L.phi0, L.q0, L.rhs, sc32(l),
-                     ops32[l], colour);
+          default: {
+            auto tile = [&](auto launch) {
+              launch(st, L.n, co, L.e, L.phi0, qv, gv, sc32(l), ops32[l], colour);
+            };
+            if (L.n < kColour32TileMin)
+              launch_k(k_smooth_colour32, nb, 256, 0, st, L.n, L.e, L.phi0, L.q0, L.rhs, sc32(l),
+                       ops32[l], colour);
+            else if (colour32_narrow(L.n))
+              tile(launch_colour32_tile<16>);
+            else
+              tile(launch_colour32_tile<32>);
+          }
         }
         if (timed) t->end(st);
       }
