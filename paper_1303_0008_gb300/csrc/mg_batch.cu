@@ -72,6 +72,13 @@ __device__ __forceinline__ int3 tile_origin(int n, long long blk) {
   return make_int3((int)(b - r * g.x) * kTileX, (int)(r % g.y) * kTileY, (int)(r / g.y) * kTileZ);
 }
 
+// Block blk of a prolongation by columns of four cells.
+__device__ __forceinline__ int3 column_block(int nc, long long blk) {
+  const dim3 g = prolong_grid(nc, 4);
+  const unsigned b = (unsigned)blk, r = b / g.x;
+  return make_int3((int)(b - r * g.x), (int)(r % g.y), (int)(r / g.y));
+}
+
 // run(f, lin) with both flags as types.
 template <typename Run>
 __device__ __forceinline__ void pick(bool f, bool lin, Run run) {
@@ -164,6 +171,11 @@ __global__ void __launch_bounds__(256) kb_fas_rhs64(const BItem* __restrict__ it
 __global__ void __launch_bounds__(256) kb_prolong64(const BItem* __restrict__ items, int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
+  if (prolong_columns(it.n / 2)) {
+    const int3 o = column_block(it.n / 2, blk);
+    prolong_column<double, double2, 4>(it.n / 2, it.cphi, it.cphihat, it.phi, o.x, o.y, o.z);
+    return;
+  }
   b_prolong_correct64(it.n / 2, it.cphi, it.cphihat, it.phi, blk);
 }
 
@@ -226,6 +238,7 @@ __global__ void __launch_bounds__(256) kb_smooth32(const BItem* __restrict__ ite
   const dim3 g = narrow ? colour32_grid<16>(it.n) : colour32_grid<32>(it.n);
   const unsigned b = (unsigned)blk, r = b / g.x;
   const int bx = (int)(b - r * g.x), by = (int)(r % g.y), bz = (int)(r / g.y);
+  // (q0 and g in colour order, as the single grids read them, gained nothing here)
   if (narrow)
     b_colour32_tile<16, false>(it.n, it.e, it.phi0, it.q0, it.rhs, s_mu, it.op32, colour, bx, by,
                                bz);
@@ -251,6 +264,11 @@ __global__ void __launch_bounds__(256) kb_fas_rhs32(const BItem* __restrict__ it
 __global__ void __launch_bounds__(256) kb_prolong32(const BItem* __restrict__ items, int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
+  if (prolong_columns(it.n / 2)) {
+    const int3 o = column_block(it.n / 2, blk);
+    prolong_column<float, float2, 4>(it.n / 2, it.ce, it.cehat, it.e, o.x, o.y, o.z);
+    return;
+  }
   b_prolong_correct32(it.n / 2, it.ce, it.cehat, it.e, blk);
 }
 
@@ -264,10 +282,12 @@ __global__ void __launch_bounds__(256) kb_coarsest_corr32(const BItem* __restric
 // Host side
 // ---------------------------------------------------------------------------
 // T_HAND: the outer residual hand-off, kHandoffCells cells per thread
+// T_PROLONG: the prolongations, by columns where they run so;
 // T_SM64, T_RR64, T_CCELL64: the FP64 colour stages, residual restrictions and right-hand
 // sides (of the level below), and T_HAND: in tiles from kTileMinSide on
 enum ListType {
-  T_SMOOTH = 0, T_RR, T_CELL, T_CCELL, T_ONE, T_HAND, T_SM64, T_RR64, T_CCELL64, T_NTYPES
+  T_SMOOTH = 0, T_RR, T_CELL, T_CCELL, T_ONE, T_HAND, T_SM64, T_RR64, T_CCELL64,
+  T_PROLONG, T_NTYPES
 };
 
 static long long blocks_of(ListType t, const BItem& it) {
@@ -287,6 +307,11 @@ static long long blocks_of(ListType t, const BItem& it) {
       return (cells / 8 + 255) / 256;
     case T_RR: return (cells / 8 + 255) / 256;
     case T_CELL: return (cells + 255) / 256;
+    case T_PROLONG: {
+      if (!prolong_columns(n / 2)) return (cells + 255) / 256;
+      const dim3 g = prolong_grid(n / 2, 4);
+      return (long long)g.x * g.y * g.z;
+    }
     case T_CCELL64:
       if (in_tiles(n / 2, it.cop)) return tile_count(n / 2);
       return (cells / 8 + 255) / 256;
@@ -516,7 +541,7 @@ struct BatchCycle {
                                                          o->coarse_drop);
     count_launches(1);
     for (int l = bs->lmax - 2; l >= 0; --l) {
-      launch(L(l, T_CELL, P_DESC), 256, kb_prolong64);
+      launch(L(l, T_PROLONG, P_DESC), 256, kb_prolong64);
       smooth64(l, o->nu_post);
     }
   }
@@ -545,7 +570,7 @@ struct BatchCycle {
                                                               o->coarse_drop);
     count_launches(1);
     for (int l = bs->lmax - 2; l >= 0; --l) {
-      launch(L(l, T_CELL, P_DESC), 256, kb_prolong32);
+      launch(L(l, T_PROLONG, P_DESC), 256, kb_prolong32);
       smooth32(l, o->nu_post);
     }
   }

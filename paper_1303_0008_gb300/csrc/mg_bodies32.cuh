@@ -762,7 +762,7 @@ __device__ __forceinline__ void b_fas_rhs32(int nc, const float* __restrict__ e_
 }
 
 // One fine cell of the trilinear prolongation of e_c - ehat_c into e_f (t indexes
-// the (2 nc)^3 fine cells).
+// the (2 nc)^3 fine cells), in the order of prolong_column.
 __device__ __forceinline__ void cell_prolong32(int nc, const float* __restrict__ e_c,
                                                const float* __restrict__ ehat_c,
                                                float* __restrict__ e_f, long long t) {
@@ -777,31 +777,11 @@ __device__ __forceinline__ void cell_prolong32(int nc, const float* __restrict__
   const int K1 = (k & 1) ? wrap_up(K0, nc) : wrap_dn(K0, nc);
   auto v = [&](int a, int b, int cc) {
     const long long q = lidx(a, b, cc, nc);
-    return e_c[q] - ehat_c[q];
+    return __fsub_rn(e_c[q], ehat_c[q]);
   };
-  const float s = 27.f * v(I0, J0, K0) + 9.f * (v(I1, J0, K0) + v(I0, J1, K0) + v(I0, J0, K1)) +
-                  3.f * (v(I1, J1, K0) + v(I1, J0, K1) + v(I0, J1, K1)) + v(I1, J1, K1);
-  e_f[t] += s * (1.f / 64.f);
-}
-
-// cell_prolong32 from the coarse correction corr_c = e_c - ehat_c formed beforehand
-// (once per coarse cell instead of once per fine cell that reads it): the same
-// values in the same sum.
-__device__ __forceinline__ void cell_prolong_corr32(int nc, const float* __restrict__ corr_c,
-                                                    float* __restrict__ e_f, long long t) {
-  const int nf = nc << 1;
-  const long long cells = (long long)nf * nf * nf;
-  if (t >= cells) return;
-  int i, j, k;
-  split3((unsigned)t, nf, i, j, k);
-  const int I0 = i >> 1, J0 = j >> 1, K0 = k >> 1;
-  const int I1 = (i & 1) ? wrap_up(I0, nc) : wrap_dn(I0, nc);
-  const int J1 = (j & 1) ? wrap_up(J0, nc) : wrap_dn(J0, nc);
-  const int K1 = (k & 1) ? wrap_up(K0, nc) : wrap_dn(K0, nc);
-  auto v = [&](int a, int b, int cc) { return corr_c[lidx(a, b, cc, nc)]; };
-  const float s = 27.f * v(I0, J0, K0) + 9.f * (v(I1, J0, K0) + v(I0, J1, K0) + v(I0, J0, K1)) +
-                  3.f * (v(I1, J1, K0) + v(I1, J0, K1) + v(I0, J1, K1)) + v(I1, J1, K1);
-  e_f[t] += s * (1.f / 64.f);
+  auto row = [&](int b, int cc) { return __fmaf_rn(3.f, v(I0, b, cc), v(I1, b, cc)); };
+  auto plane = [&](int cc) { return __fmaf_rn(3.f, row(J0, cc), row(J1, cc)); };
+  e_f[t] = __fmaf_rn(__fmaf_rn(3.f, plane(K0), plane(K1)), 1.f / 64.f, e_f[t]);
 }
 
 __device__ __forceinline__ void b_prolong_correct32(int nc, const float* __restrict__ e_c,

@@ -151,94 +151,14 @@ __global__ void __launch_bounds__(256) k_restrict_defects64(
   b_restrict_defects64(nf, phi, din, gin, phi_c, phihat_c, rd_c, partials, blockIdx.x);
 }
 
-// The prolongation of a large level by columns: a thread takes KZ coarse cells above one
-// another and their 8 KZ children, the CTA 32 x 8 columns.  A coarse plane's corrections
-// are formed once in shared memory, interpolated along x and y once (10 multiply-adds per
-// coarse cell) and used for the planes of children above and below: 3.7 FP64 instructions
-// per fine cell instead of 11 (19 with the corrections formed by each of their readers).
-// At 300^3 the kernel takes 223 instead of 873 us; in the FP64 solve of 512^3
-// the finest one 1.0 instead of 2.4 ms.  The FP64 pipe still bounds it.
+// The prolongation of a large level by columns (prolong_column).
 template <int KZ>
 __global__ void __launch_bounds__(256) k_prolong_column64(int nc, const double* __restrict__ phi_c,
                                                           const double* __restrict__ phihat_c,
                                                           double* __restrict__ phi_f) {
   PdlScope pdl_scope;
-  constexpr int W = 34, H = 10;
-  __shared__ double e[2][W * H];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int I0 = (int)blockIdx.x * 32, J0 = (int)blockIdx.y * 8, K0 = (int)blockIdx.z * KZ;
-  auto wrap = [nc](int v) { return v < 0 ? v + nc : (v >= nc ? v - nc : v); };
-  int at[2];  // this thread's cells of a plane of the CTA's tile
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int q = threadIdx.x + 256 * r, y = q / W;
-    at[r] = wrap(J0 - 1 + y) * nc + wrap(I0 - 1 + q - W * y);
-  }
-  auto load = [&](int K, double* t) {
-    const long long p = (long long)wrap(K) * nc * nc;
-    t[threadIdx.x] = phi_c[p + at[0]] - phihat_c[p + at[0]];
-    if (threadIdx.x < W * H - 256)
-      t[threadIdx.x + 256] = phi_c[p + at[1]] - phihat_c[p + at[1]];
-  };
-  // (y side, x side) of the column's cell in a plane: towards -y or +y, -x or +x
-  auto interpolate = [&](const double* t, double (&b)[4]) {
-    double a[3][2];
-#pragma unroll
-    for (int y = 0; y < 3; ++y) {
-      const double* r = t + (w + y) * W + lane + 1;
-      a[y][0] = fma(3.0, r[0], r[-1]);
-      a[y][1] = fma(3.0, r[0], r[1]);
-    }
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      b[x] = fma(3.0, a[1][x], a[0][x]);
-      b[2 + x] = fma(3.0, a[1][x], a[2][x]);
-    }
-  };
-  double lo[4], mid[4], up[4];
-  load(K0 - 1, e[0]);
-  load(K0, e[1]);
-  __syncthreads();
-  interpolate(e[0], lo);
-  interpolate(e[1], mid);
-  __syncthreads();
-  const int I = I0 + lane, J = J0 + w, nf = 2 * nc;
-  const bool in = I < nc && J < nc;
-#pragma unroll 1
-  for (int s = 0; s < KZ && K0 + s < nc; ++s) {
-    const int K = K0 + s;
-    double* t = e[s & 1];
-    load(K + 1, t);
-    double2 v[4];
-    double2* f = reinterpret_cast<double2*>(phi_f + lidx(2 * I, 2 * J, 2 * K, nf));
-    const long long row = nf / 2, plane = (long long)nf * nf / 2;  // in pairs
-    if (in) {
-      v[0] = f[0];
-      v[1] = f[row];
-      v[2] = f[plane];
-      v[3] = f[plane + row];
-    }
-    __syncthreads();
-    interpolate(t, up);
-    if (in) {
-#pragma unroll
-      for (int y = 0; y < 2; ++y) {
-        v[y].x = fma(fma(3.0, mid[2 * y], lo[2 * y]), 1.0 / 64.0, v[y].x);
-        v[y].y = fma(fma(3.0, mid[2 * y + 1], lo[2 * y + 1]), 1.0 / 64.0, v[y].y);
-        v[2 + y].x = fma(fma(3.0, mid[2 * y], up[2 * y]), 1.0 / 64.0, v[2 + y].x);
-        v[2 + y].y = fma(fma(3.0, mid[2 * y + 1], up[2 * y + 1]), 1.0 / 64.0, v[2 + y].y);
-      }
-      f[0] = v[0];
-      f[row] = v[1];
-      f[plane] = v[2];
-      f[plane + row] = v[3];
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      lo[q] = mid[q];
-      mid[q] = up[q];
-    }
-  }
+  prolong_column<double, double2, KZ>(nc, phi_c, phihat_c, phi_f, (int)blockIdx.x,
+                                      (int)blockIdx.y, (int)blockIdx.z);
 }
 
 // One block: reduce the partials in a fixed order and publish the scalars.
@@ -528,20 +448,15 @@ void launch_fas_rhs64(cudaStream_t st, int nc, const double* phi_c, const double
   count_launches(1);
 }
 
-// By columns from nc = 48 on (fine side 96, where CTAs of four cells deep columns reach
-// most SMs); deeper columns once they leave four CTAs per SM.  The columns' loads of pairs
-// need a 16-byte aligned field.
+// By columns where prolong_columns says so.  Their loads of pairs need a 16-byte aligned
+// field.
 void launch_prolong_correct64(cudaStream_t st, int nc, const double* phi_c,
                               const double* phihat_c, double* phi_f) {
   const long long cells = 8LL * nc * nc * nc;
-  const unsigned bx = blocks_for(nc, 32), by = blocks_for(nc, 8);
-  if (nc >= 48 && reinterpret_cast<uintptr_t>(phi_f) % 16 == 0) {
-    if ((long long)bx * by * blocks_for(nc, 8) >= 608)
-      launch_k(k_prolong_column64<8>, dim3(bx, by, blocks_for(nc, 8)), 256, 0, st, nc, phi_c,
-               phihat_c, phi_f);
-    else
-      launch_k(k_prolong_column64<4>, dim3(bx, by, blocks_for(nc, 4)), 256, 0, st, nc, phi_c,
-               phihat_c, phi_f);
+  if (prolong_columns(nc) && reinterpret_cast<uintptr_t>(phi_f) % 16 == 0) {
+    const int kz = prolong_depth(nc);
+    launch_k(kz == 8 ? k_prolong_column64<8> : k_prolong_column64<4>, prolong_grid(nc, kz), 256, 0,
+             st, nc, phi_c, phihat_c, phi_f);
   } else {
     const int tpb = tpb_for(cells);
     launch_k(k_prolong_correct64, blocks_for(cells, tpb), tpb, 0, st, nc, phi_c, phihat_c, phi_f);

@@ -272,22 +272,14 @@ __global__ void __launch_bounds__(256) k_prolong_correct32(int nc, const float* 
   b_prolong_correct32(nc, e_c, ehat_c, e_f, blockIdx.x);
 }
 
-// ehat_c <- e_c - ehat_c (R e is not needed after the prolongation), then the
-// prolongation from it: the subtraction once per coarse cell instead of once per fine
-// cell that reads it, on levels from kCorrectionMinFine fine cells on.
-constexpr long long kCorrectionMinFine = 128LL * 128 * 128;
-
-__global__ void __launch_bounds__(256) k_correction32(long long cells, const float* __restrict__ e_c,
-                                                      float* __restrict__ ehat_c) {
+// The same by columns (prolong_column).
+template <int KZ>
+__global__ void __launch_bounds__(256) k_prolong_column32(int nc, const float* __restrict__ e_c,
+                                                          const float* __restrict__ ehat_c,
+                                                          float* __restrict__ e_f) {
   PdlScope pdl_scope;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < cells) ehat_c[t] = e_c[t] - ehat_c[t];
-}
-
-__global__ void __launch_bounds__(256) k_prolong_corr32(int nc, const float* __restrict__ corr_c,
-                                                        float* __restrict__ e_f) {
-  PdlScope pdl_scope;
-  cell_prolong_corr32(nc, corr_c, e_f, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+  prolong_column<float, float2, KZ>(nc, e_c, ehat_c, e_f, (int)blockIdx.x, (int)blockIdx.y,
+                                    (int)blockIdx.z);
 }
 
 // Coarsest inner level in one CTA, in FP32: sweeps of N(e) = g + mu until the
@@ -350,7 +342,9 @@ void mixed_release(Domain* d) {
   d->mixed_ready = false;
 }
 
-static mg_status mixed_prepare(Domain* d) {
+// colour_order: also q0 and g in colour order on the finest level, without which its colour
+// stages read the natural arrays (so a failed allocation of these is no error).
+static mg_status mixed_prepare(Domain* d, bool colour_order) {
   if (d->mixed_ready) return MG_OK;
   bool ok = true;
   for (int l = 0; l < d->nlev; ++l) {
@@ -362,10 +356,6 @@ static mg_status mixed_prepare(Domain* d) {
     ok = ok && cudaMalloc(&L.rhs, b) == cudaSuccess;
     if (l > 0) ok = ok && cudaMalloc(&L.ehat, b) == cudaSuccess;
     if (sweep32_eligible(L.n)) ok = ok && cudaMalloc(&L.e2, b) == cudaSuccess;
-    if (l == 0 && L.n >= 64) {
-      ok = ok && cudaMalloc(&L.q0c, b) == cudaSuccess;
-      ok = ok && cudaMalloc(&L.rhsc, b) == cudaSuccess;
-    }
   }
   ok = ok && cudaMalloc(&d->d_flags, 4 * sizeof(int)) == cudaSuccess;
   ok = ok && cudaMallocHost(&d->h_flags, 4 * sizeof(int)) == cudaSuccess;
@@ -374,6 +364,15 @@ static mg_status mixed_prepare(Domain* d) {
     mixed_release(d);
     set_error("device allocation failed (mixed precision arrays)");
     return MG_ENOMEM;
+  }
+  Level& F = d->lv[0];
+  if (colour_order && F.n >= 64) {
+    const size_t b = (size_t)F.cells * sizeof(float);
+    if (cudaMalloc(&F.q0c, b) != cudaSuccess || cudaMalloc(&F.rhsc, b) != cudaSuccess) {
+      cudaFree(F.q0c);
+      F.q0c = F.rhsc = nullptr;
+      cudaGetLastError();
+    }
   }
   static bool attr = false;
   if (!attr) {
@@ -387,7 +386,7 @@ static mg_status mixed_prepare(Domain* d) {
   return MG_OK;
 }
 
-mg_status mixed_prepare_domain(Domain* d) { return mixed_prepare(d); }
+mg_status mixed_prepare_domain(Domain* d) { return mixed_prepare(d, false); }
 
 struct CycleMixed {
   Domain* d;
@@ -571,10 +570,10 @@ struct CycleMixed {
     launch_k(k_fas_rhs32, nblk(C.cells, 256), 256, 0, st, C.n, C.e, C.phi0, C.q0, C.rhs, ops32[l + 1],
                                                      sc32(l), sc32(l + 1));
     inner(l + 1);
-    if (L.cells >= kCorrectionMinFine) {
-      launch_k(k_correction32, nblk(C.cells, 256), 256, 0, st, C.cells, C.e, C.ehat);
-      launch_k(k_prolong_corr32, nblk(L.cells, 256), 256, 0, st, C.n, (const float*)C.ehat, L.e);
-      count_launches(1);
+    if (prolong_columns(C.n)) {
+      const int kz = prolong_depth(C.n);
+      launch_k(kz == 8 ? k_prolong_column32<8> : k_prolong_column32<4>, prolong_grid(C.n, kz), 256,
+               0, st, C.n, C.e, C.ehat, L.e);
     } else {
       launch_k(k_prolong_correct32, nblk(L.cells, 256), 256, 0, st, C.n, C.e, C.ehat, L.e);
     }
@@ -620,7 +619,7 @@ struct CycleMixed {
 
 mg_status mixed_solve(Domain* d, const mg_options& o, cudaStream_t st, const OpConst64* ops,
                       int branch, double alpha, double kappa, double tol, mg_solve_stats* s) {
-  mg_status ps = mixed_prepare(d);
+  mg_status ps = mixed_prepare(d, true);
   if (ps != MG_OK) return ps;
   std::vector<OpConst32> ops32(d->nlev);
   for (int l = 0; l < d->nlev; ++l) ops32[l] = make_op32(d->lv[l].n, alpha, branch);
