@@ -294,14 +294,29 @@ __device__ __forceinline__ float gal_offdiag(const float* __restrict__ J, const 
                                              int k) {
   constexpr int BC = B * B * B;
   const int t = i + B * (j + B * k);
-  float sum = 0.0f;
+  // The patches that hold the 26 neighbours, then their values and the row, then the sum:
+  // each group of loads is under way at once.  (With the test for a missing patch between
+  // each pair of dependent loads, a colour of 16384 patches took 9.7 us at B = 2 and 19.0 us
+  // at B = 4; now 5.8 and 13.4 us.)
+  int at[27];
+#pragma unroll
+  for (int o = 0; o < 27; ++o) {
+    const int x = i + o % 3 - 1, y = j + (o / 3) % 3 - 1, z = k + o / 9 - 1;
+    const bool in = (unsigned)x < (unsigned)B && (unsigned)y < (unsigned)B && (unsigned)z < (unsigned)B;
+    const int q = in ? p : nbr[p * 27 + gal_region(x, y, z, B)];
+    at[o] = q < 0 ? -1 : q * BC + gal_wrap(x, B) + B * (gal_wrap(y, B) + B * gal_wrap(z, B));
+  }
+  float v[27], a[27];
 #pragma unroll
   for (int o = 0; o < 27; ++o) {
     if (o == 13) continue;
-    const int ox = o % 3 - 1, oy = (o / 3) % 3 - 1, oz = o / 9 - 1;
-    const float a = J[((long long)p * 27 + o) * BC + t];
-    sum = fmaf(a, gal_fetch<B>(e, nbr, p, i + ox, j + oy, k + oz), sum);
+    v[o] = at[o] < 0 ? 0.0f : e[at[o]];
+    a[o] = J[((long long)p * 27 + o) * BC + t];
   }
+  float sum = 0.0f;
+#pragma unroll
+  for (int o = 0; o < 27; ++o)
+    if (o != 13) sum = fmaf(a[o], v[o], sum);
   return sum;
 }
 
