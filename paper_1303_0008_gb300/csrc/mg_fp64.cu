@@ -485,7 +485,8 @@ void launch_restrict64(cudaStream_t st, int nc, const double* fine, double* coar
 
 void launch_affine64(cudaStream_t st, long long cells, const double* x, double* out, double a,
                      double b, double c3, int floor, unsigned long long* floored) {
-  launch_k(k_affine64, blocks_for(cells, 256), 256, 0, st, cells, x, out, a, b, c3, floor, floored);
+  launch_k(k_affine64, blocks_for(cells, 256 * kAffineCells), 256, 0, st, cells, x, out, a, b, c3,
+           floor, floored);
   count_launches(1);
 }
 

@@ -122,3 +122,70 @@ def test_other_modes_in_tiles(n, alpha):
     k2 = 0.0 if abs(alpha) < 1e-4 else abs(2 / (8 / 3 * alpha))
     tol = 8 * 2.0 ** -53 * (np.abs(phi).max() + float(np.abs(D).max() + k2) / (n * n))
     assert np.abs(got - want)[first].max() <= tol
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_batch_in_tiles_has_the_bits_of_single_grids(mixed):
+    """Sides below, at and above the first that runs in tiles."""
+    from paper_1303_0008_gb300 import inputs as I
+
+    opt = dict(prec=mg.MG_MIXED if mixed else mg.MG_FP64)
+    specs = [(n, I.lognormal_delta(n, 1.5, n), s * I.alpha_kappa_for_rv(8.0), s)
+             for n, s in ((96, 1.0), (112, -1.0), (128, 1.0), (160, 1.0))]
+    g = mg.mg_create_batch([n for n, *_ in specs], mg.options(**opt))
+    try:
+        for k, (_, d, _, _) in enumerate(specs):
+            mg.mg_set_density(g, 0, k, d)
+        mg.mg_solve_batch(g, [0] * len(specs), [a for _, _, a, _ in specs],
+                          [s for *_, s in specs], 1e-8)
+        batch = [mg.mg_get_field(g, 0, k, np.empty((n,) * 3)) for k, (n, *_) in enumerate(specs)]
+    finally:
+        mg.mg_destroy_grid(g)
+    for (n, d, a, s), got in zip(specs, batch):
+        h = mg.mg_create_grid(n, mg.options(**opt))
+        try:
+            mg.mg_set_density(h, 0, -1, d)
+            mg.mg_solve(h, 0, a, s, 1e-8)
+            assert np.array_equal(mg.mg_get_field(h, 0, -1, np.empty((n,) * 3)), got)
+        finally:
+            mg.mg_destroy_grid(h)
+
+
+@pytest.mark.parametrize("n", [94, 96, 100, 134, 258])
+def test_prolongation_by_columns(n):
+    """Against the tensor product of (3/4, 1/4), and a field that is not 16-byte aligned,
+    which goes cell by cell, bit for bit."""
+    rng = np.random.default_rng(n)
+    h = n // 2
+    c, r = (torch.from_numpy(rng.standard_normal((h, h, h))).cuda() for _ in range(2))
+    f = torch.from_numpy(rng.standard_normal((n, n, n))).cuda()
+    want = c - r
+    for axis in range(3):
+        lo, hi = want.roll(1, axis), want.roll(-1, axis)
+        want = torch.stack((0.25 * lo + 0.75 * want, 0.75 * want + 0.25 * hi), dim=axis + 1)
+        want = want.flatten(axis, axis + 1)
+    want = want + f
+    got = f.clone()
+    mg.mg_op_prolong_correct(n, c, r, got)
+    odd = torch.empty(n ** 3 + 1, dtype=torch.float64, device="cuda")[1:].view(n, n, n)
+    odd.copy_(f)
+    mg.mg_op_prolong_correct(n, c, r, odd)
+    torch.cuda.synchronize()
+    # three multiply-adds and one more, of values up to max|c - r| and max|f|
+    tol = 8 * 2.0 ** -53 * float((c - r).abs().max() + f.abs().max())
+    assert float((got - want).abs().max()) <= tol
+    assert torch.equal(got, odd)
+
+
+@pytest.mark.parametrize("n", [32, 48, 128])
+def test_force_factor(n):
+    """-(n/4) times the difference, rounded once: by the exponent where n is a power of two."""
+    rng = np.random.default_rng(n)
+    phi = rng.standard_normal((n, n, n)) * np.exp(rng.uniform(-650, 300, (n, n, n)))
+    phi[:2] = 0.0
+    out = torch.empty((3, n, n, n), dtype=torch.float64, device="cuda")
+    mg.mg_op_force(n, torch.from_numpy(phi).cuda(), out)
+    torch.cuda.synchronize()
+    for a, axis in enumerate((2, 1, 0)):
+        want = -0.25 * n * (np.roll(phi, -1, axis) - np.roll(phi, 1, axis))
+        assert np.array_equal(out[a].cpu().numpy(), want)
