@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(256) k_residual64(int n, const double* __restr
 
 // The same for levels of many tiles, one partial per tile.
 template <bool LIN>
-__global__ void __launch_bounds__(256, 3) k_residual_tile64(int n, const double* __restrict__ phi,
+__global__ void __launch_bounds__(256, 4) k_residual_tile64(int n, const double* __restrict__ phi,
                                                             const double* __restrict__ src,
                                                             const double* __restrict__ f,
                                                             double* __restrict__ dout,
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(256) k_fas_rhs64(int nc, const double* __restr
 
 // The same for levels of many tiles.
 template <bool LIN>
-__global__ void __launch_bounds__(256, 3) k_fas_rhs_tile64(int nc, const double* __restrict__ phi_c,
+__global__ void __launch_bounds__(256, 4) k_fas_rhs_tile64(int nc, const double* __restrict__ phi_c,
                                                            const double* __restrict__ src_c,
                                                            double* __restrict__ f_c, OpConst64 c,
                                                            const LevelScalars* __restrict__ fine_sc,

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256) k_residual_handoff64(int n, const double*
 
 // The same for levels of many tiles, one partial per tile.
 template <bool LIN>
-__global__ void __launch_bounds__(256, 3) k_handoff_tile64(int n, const double* __restrict__ phi,
+__global__ void __launch_bounds__(256, 4) k_handoff_tile64(int n, const double* __restrict__ phi,
                                                            const double* __restrict__ src,
                                                            OpConst64 c,
                                                            const LevelScalars* __restrict__ sc,

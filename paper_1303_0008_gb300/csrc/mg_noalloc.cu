@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kNoAllocThreads) k_residual64_noalloc(
 
 // The same for grids of many tiles, one partial per tile.
 template <bool LIN>
-__global__ void __launch_bounds__(256, 3) k_residual_tile64_noalloc(
+__global__ void __launch_bounds__(256, 4) k_residual_tile64_noalloc(
     int n, const double* __restrict__ phi, const double* __restrict__ delta, double a, double b,
     const double* __restrict__ f, double* __restrict__ dout, OpConst64 c,
     NoAllocScratch* __restrict__ scratch) {

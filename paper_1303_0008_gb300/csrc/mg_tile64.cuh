@@ -41,7 +41,7 @@ __host__ __device__ inline unsigned tile_count(int n) {
 
 // Whether a level runs in tiles: its operator in the square-root or the linear form.  The
 // others (a splitting constant of its own, |alpha| < 1e-4) divide and would cost the tile
-// kernels the registers of a fourth CTA per SM; their cells go one by one.
+// kernels the registers of their fourth CTA per SM; their cells go one by one.
 __host__ __device__ inline bool in_tiles(int n, const OpConst64& c) {
   return n >= kTileMinSide && (c.mode == OP_SQRT || c.mode == OP_LINEAR);
 }
@@ -407,8 +407,10 @@ __device__ __forceinline__ bool tile_defect(const long long* q, const TilePlane&
                              (long long)(up.dx - lo.dx), (long long)(up.dy - lo.dy)};
     N = fix_quad(a, cc, sh, tq);
   }
-  bool bad = tq == 0 || ((tile_mag((long long)mid.c) << 3 | tq) < (1u << 24) &&
-                         tile_small(q, 0, -1, 1));
+  const unsigned ls = (unsigned)(fix_hi(lap) >> 31);
+  const u64 lm = ((u64)lap ^ fix_words(ls, ls)) - fix_words(ls, ls);
+  bool bad = min((unsigned)(lm >> 32), tq) == 0 ||
+             ((tile_mag((long long)mid.c) << 3 | tq) < (1u << 24) && tile_small(q, 0, -1, 1));
   double D = src;
   qd = 1.0;
   if (!LIN) {
@@ -416,14 +418,16 @@ __device__ __forceinline__ bool tile_defect(const long long* q, const TilePlane&
     bad = bad || !fix_normal(qd);
     D = fma(c.k2s, sqrt_fix_normal(qd), -c.k2);
   }
-  d = fma(fix_signed(lap, FixRef{0, ue + 1, false}), c.inv_h2, -D);
+  d = fma(fix_double_top(lm, ue + 1, ls & 0x80000000u), c.inv_h2, -D);
   return !bad;
 }
 
-// The defect kernels, 512^3: residual 13.1 -> 1.94 ms, residual with restriction 10.5 ->
-// 2.46 ms, hand-off to FP32 10.5 -> 3.38 ms (256^3 residual 1646 -> 253 us).  Per cell three
-// to five FP64 instructions remain (the FP64 pipe is about half busy), and three CTAs per SM
-// leave latency in sight; four, at 64 registers, spilled and took 3 % longer.
+// The defect kernels, 512^3: residual 13.1 -> 1.65 ms, residual with restriction 10.5 ->
+// 2.32 ms, hand-off to FP32 10.5 -> 3.11 ms (256^3 residual 1646 -> 220 us).  Per cell three
+// to five FP64 instructions remain (the FP64 pipe is about half busy) beside some 430 others,
+// two thirds of the issue slots.  Four CTAs per SM at 64 registers against three at 80:
+// residual 1.65 against 1.80 ms, hand-off 3.11 against 3.28 ms; the restriction, which keeps
+// two columns at once, is fastest at two.
 //
 // Visit every cell of the tile at (x0, y0, z0): cell(id, i, j, k, defect, q, guard) with
 // src(id) its source term.  A thread takes two columns of eight cells, side by side in y,
