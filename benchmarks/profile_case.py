@@ -7,7 +7,7 @@ Runs a single periodic solve (default sigma 1.5, seed 1302) to 1e-8 on cuda:0, o
 --six the six solves of one step of the benchmark, and prints the statistics of
 each solve as one JSON line.  --case selects the other kernel families: a
 refined hierarchy, the batched solves, or particle assignment with refinement.  Meant to be run under a profiler with a kernel
-filter (for instance `ncu -k regex:k_smooth_colour64 -s 4 -c 3 ...`): at n = 256
+filter (for instance `ncu -k regex:k_smooth_tile64 -s 4 -c 3 ...`): at n = 256
 every FP64 array of the finest level is 134 MB, larger than the 126 MB L2, so
 DRAM counters describe HBM traffic.
 """
