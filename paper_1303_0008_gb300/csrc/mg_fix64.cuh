@@ -4,21 +4,27 @@
 // holds its scheduler's FP64 unit for 64 cycles; an integer one takes 1 to 2.  A cell of
 // the operator needs 18 neighbours, 14 additions, six squares and a square root, about 33
 // FP64 instructions.  Here everything but three fused multiply-adds runs in 64-bit
-// integers, with no step less exact than its FP64 form:
+// integers:
 //   fix_align   the neighbours as integers of one unit.  Values of one sign and binade
 //               (the usual case: the field varies by a few percent over a stencil) need
 //               no conversion at all: their bit patterns differ by exactly the
 //               differences of their significands.  Values of one sign and near
 //               binades are shifted up, exactly; others are shifted to the largest
-//               exponent, with 6 or 7 more bits below.
-//   sums        exact (FP64 rounds each to half a unit in the last place of the field).
-//   fix_quad    the quadratic form of Sigma_d as a 62-bit integer, error below 2^-53.
-//   sqrt_fix    square root to about 2^-61 from the FP32 reciprocal square root and two
-//               exact integer residuals.
+//               exponent, with 6 or 7 more bits below, and cut off there (2^-58 or 2^-59 of
+//               the largest).
+//   sums        exact sums of those integers (FP64 rounds each to half a unit in its last
+//               place), so exact sums of the values in the first two forms.
+//   fix_quad    the quadratic form of Sigma_d as a 62-bit integer, error below 2^-53 of it;
+//               where all second differences are below 2^32 units it counts in 2^4 squared
+//               units and is off by up to four of those.
+//   sqrt_fix    square root to about 2^-61 (half a unit in the last place and 2^-8 of one at
+//               most) from the FP32 reciprocal square root and two exact integer residuals.
 //   fix_double  back to FP64, rounded once.
+// A cell's error is below that of its FP64 form (tests/test_tile_accuracy.py: 0.5 to 0.95 of
+// it, rms).
 // Cells whose values have no such form (all zero, infinities, NaN, exponents whose
-// squares leave the FP64 range) keep the FP64 code.  Every function depends on its arguments alone, so
-// all kernels that update a cell give the same bits.
+// squares leave the FP64 range) keep the FP64 code.  Every function depends on its arguments
+// alone, so all kernels that update a cell give the same bits.
 #pragma once
 
 #include <cstdint>
@@ -222,7 +228,8 @@ MG_HD double fix_signed(long long v, const FixRef& r) {
 // Sum a^2 + (3/8) sum c^2 = N 2^(64 - 2 sh) of integers below 2^62 (top: their high words
 // or-ed, signs removed): each value is shifted so that the largest lies in [2^61, 2^62)
 // and split as h 2^32 + l with -2^31 <= l < 2^31; h^2 and h l are exact, l^2 (a quarter
-// of a unit of N at most) is left out.
+// of a unit of N at most) is left out.  The shift ends at 30: N of (1, 1, 0) is 0, of
+// (3, 3, 0) 16 for 18.
 MG_HD unsigned long long fix_quad(const long long (&a)[3], const long long (&c)[3], int& sh,
                                   unsigned& top) {
   top = 0;
@@ -281,6 +288,36 @@ MG_HD double sqrt_fix_normal(double q) {
   return fix_pack((unsigned)t, (unsigned)s0 + (unsigned)(t >> 32),
                   ((e - 1023 - odd) >> 1) + 1022, 0);
 }
+
+// x >> d for any d >= 0, with copies of the sign from 63 on.
+MG_HD long long fix_sar(long long x, int d) {
+#ifdef __CUDA_ARCH__
+  asm("shr.s64 %0, %0, %1;" : "+l"(x) : "r"(d));
+  return x;
+#else
+  return x >> (d < 63 ? d : 63);
+#endif
+}
+
+// b as an integer of the unit 2^-59 of a tile (mg_tile64.cuh) whose exponent field (in place)
+// is em, rounded to nearest: the significand up by 8 bits, with its sign (the complement: one
+// unit off), down by the difference of the exponents to twice the unit's resolution, and the
+// last bit rounded, which takes the complement's unit back too.
+MG_HD long long tile_convert(long long b, int em) {
+  const int h = fix_hi(b);
+  const unsigned s = (unsigned)(h >> 31);
+  const unsigned lo = (unsigned)b, mh = (unsigned)((h & 0xfffff) | 0x100000);
+  const long long t = fix_sar((long long)fix_words((lo << 8) ^ s, fix_shl_hi(lo, mh, 8) ^ s),
+                              (em - (h & 0x7ff00000)) >> 20);
+  return (t + 1) >> 1;
+}
+
+// The high word of a tile value's magnitude, and the bounds that one of the six across a cell's
+// faces has to reach, or the unit would be too coarse for the cell: 2^-7 of the tile's range
+// for an update, where six rounded values count a sixth each, and 2^-6 for a defect (there
+// the centre's may do as well), to which the centre adds six times its own rounding.
+MG_HD unsigned tile_mag(long long v) { return (unsigned)(fix_hi(v) ^ (fix_hi(v) >> 31)); }
+constexpr unsigned kTileSmall = 1u << 21, kTileSmallDefect = 1u << 22;
 
 #ifdef __CUDACC__
 static __device__ __noinline__ float fix_to_float_rare(double x) { return (float)x; }

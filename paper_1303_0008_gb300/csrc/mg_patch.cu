@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(128) k_patch_smooth_fix(double* __restrict__ p
     unsigned long long N;
     int sh;
     unsigned tq;
-    good = patch_forms<LIN>(S.v + q, face, N, sh, tq);
+    good = patch_forms<LIN>(S.v + q, kTileSmall, face, N, sh, tq);
     double acc;
     if (LIN) {
       acc = fma(-c.h2_6, sv, s_c);
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(128) k_patch_residual_restrict_fix(
       unsigned long long N;
       int sh;
       unsigned tq;
-      good = patch_forms<LIN>(S.v + q, face, N, sh, tq);
+      good = patch_forms<LIN>(S.v + q, kTileSmallDefect, face, N, sh, tq);
       double D = sv;
       if (!LIN) {
         const double qd = fma(c.e1, fix_double(N, 64 - 2 * sh + 2 * ue), sv);

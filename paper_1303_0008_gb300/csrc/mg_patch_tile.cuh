@@ -137,9 +137,9 @@ __device__ __forceinline__ bool patch_load(int p, const double* __restrict__ phi
 
 // The sums of the cell at q of the block: face sum, the form N 2^(64 - 2 sh) (0 with LIN)
 // and a bound of its terms.  False: the block's unit does not resolve the stencil as FP64
-// would.
+// would (`bound`: kTileSmall or kTileSmallDefect).
 template <bool LIN>
-__device__ __forceinline__ bool patch_forms(const long long* q, long long& face,
+__device__ __forceinline__ bool patch_forms(const long long* q, unsigned bound, long long& face,
                                             unsigned long long& N, int& sh, unsigned& tq) {
   typedef unsigned long long u64;
   constexpr int Y = 10, Z = 100;
@@ -158,9 +158,9 @@ __device__ __forceinline__ bool patch_forms(const long long* q, long long& face,
     N = fix_quad(a, c, sh, tq);
   }
   if (tq == 0) return false;
-  if ((tile_mag(face) | tq) >= (1u << 24)) return true;
+  if ((tile_mag(face) | tq) >= 8 * bound) return true;
   return (tile_mag(q[1]) | tile_mag(q[-1]) | tile_mag(q[Y]) | tile_mag(q[-Y]) | tile_mag(q[Z]) |
-          tile_mag(q[-Z])) >= (1u << 21);
+          tile_mag(q[-Z])) >= bound;
 }
 
 // The stencil of the cell at place q of the ghosted block in FP64, from memory.

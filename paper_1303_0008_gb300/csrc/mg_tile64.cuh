@@ -5,11 +5,19 @@
 // stencils in ten cross a binade of the field or its sign.  A CTA therefore loads a tile
 // of 32 x 16 x 8 cells and its shell (34 x 18 x 10 = 6120 values, 49 KB, four CTAs per
 // SM), finds the largest exponent, and converts each value once, to a unit 2^-59 of it.
-// Then no cell converts anything: 1.5 conversions per cell instead of 18 or 19.
+// Then no cell converts anything: 1.5 conversions per cell in the kernels that visit every
+// cell and 4.5 per updated cell in a colour stage (4590 values for 1024 cells), instead of 18
+// or 19.
 //
-// What is cut off below the unit is less than FP64 additions lose as long as the stencil
-// holds a value within 2^-7 of the tile's largest; tile_small finds the others (cells at a
-// zero of the field in a steep tile), which take their values from memory.
+// Values within 2^-7 of the tile's largest keep all their bits; the others are rounded to the
+// unit.  That loses less than FP64 additions do as long as one of the six neighbours
+// across a face reaches 2^-7 of the tile's largest (2^-6 for a defect); tile_small finds the
+// other cells (those at a zero of the field in a steep tile), which take their values from
+// memory.  In units of
+// 2^-53 of an update's largest term, the error of a cell (rms and worst of 160000) where
+// 1.07 and 5.3 are FP64's: 0.88 and 4.2 on noise whose amplitude falls as exp(-0.15 i - 0.1 j)
+// through the tile (with the values cut off instead of rounded 1.14 and 6.5), 0.89 and 3.8 on
+// noise of one amplitude.
 // Tiles without such a unit (infinities, NaN, extreme exponents) go cell by cell too.
 #pragma once
 
@@ -60,17 +68,6 @@ struct TileShared {
   int em[8];
   double scalar;
 };
-
-// b as an integer of the unit 2^-59 of a tile whose exponent field (in place) is em: the
-// significand up by 7 bits, with its sign (the complement: one unit off), down by the
-// difference of the exponents.
-__device__ __forceinline__ long long tile_convert(long long b, int em) {
-  const int h = fix_hi(b);
-  const int d = min((em - (h & 0x7ff00000)) >> 20, 63);
-  const unsigned s = (unsigned)(h >> 31);
-  const unsigned lo = (unsigned)b, mh = (unsigned)((h & 0xfffff) | 0x100000);
-  return (long long)fix_words((lo << 7) ^ s, fix_shl_hi(lo, mh, 7) ^ s) >> d;
-}
 
 // The largest high word of |values|, read as FP32 numbers (their order is that of the
 // words; NaN patterns, from exponent field 0x7f8 on, win).
@@ -214,15 +211,13 @@ __device__ __forceinline__ bool tile_load(int n, const double* __restrict__ phi,
   return true;
 }
 
-// Whether no value around the cell reaches 2^-7 of the tile's range (row[o]: its place,
-// row[l], row[r]: its neighbours in x), so that FP64 could resolve the stencil better.
-__device__ __forceinline__ unsigned tile_mag(long long v) {
-  return (unsigned)(fix_hi(v) ^ (fix_hi(v) >> 31));
-}
-__device__ __forceinline__ bool tile_small(const long long* row, int o, int l, int r) {
+// Whether no value around the cell reaches `bound` (kTileSmall), so that FP64 could resolve
+// the stencil better (row[o]: its place, row[l], row[r]: its neighbours in x).
+__device__ __forceinline__ bool tile_small(const long long* row, int o, int l, int r,
+                                           unsigned bound) {
   return (tile_mag(row[l]) | tile_mag(row[r]) | tile_mag(row[o + kTileRow]) |
           tile_mag(row[o - kTileRow]) | tile_mag(row[o + kTilePlane]) |
-          tile_mag(row[o - kTilePlane])) < (1u << 21);
+          tile_mag(row[o - kTilePlane])) < bound;
 }
 
 // A colour stage on the tile at (x0, y0, z0) (256 threads): four cells per thread, on
@@ -292,7 +287,7 @@ __device__ __forceinline__ void b_smooth_tile64(int n, double* __restrict__ phi,
       const unsigned fs = (unsigned)(fix_hi(face) >> 31);
       const u64 fm = ((u64)face ^ fix_words(fs, fs)) - fix_words(fs, fs);
       const unsigned ft = (unsigned)(fm >> 32);
-      bool bad = min(ft, tq) == 0 || ((ft | tq) < (1u << 24) && tile_small(row, o, l, l + 1));
+      bool bad = min(ft, tq) == 0 || ((ft | tq) < 8 * kTileSmall && tile_small(row, o, l, l + 1, kTileSmall));
       double acc = F ? fma(fv, -c.h2_6, s_c) : s_c;
       if (LIN) {
         acc = fma(-c.h2_6, sv, acc);
@@ -410,7 +405,8 @@ __device__ __forceinline__ bool tile_defect(const long long* q, const TilePlane&
   const unsigned ls = (unsigned)(fix_hi(lap) >> 31);
   const u64 lm = ((u64)lap ^ fix_words(ls, ls)) - fix_words(ls, ls);
   bool bad = min((unsigned)(lm >> 32), tq) == 0 ||
-             ((tile_mag((long long)mid.c) << 3 | tq) < (1u << 24) && tile_small(q, 0, -1, 1));
+             ((tile_mag((long long)mid.c) << 3 | tq) < 8 * kTileSmallDefect &&
+              tile_small(q, 0, -1, 1, kTileSmallDefect));
   double D = src;
   qd = 1.0;
   if (!LIN) {
