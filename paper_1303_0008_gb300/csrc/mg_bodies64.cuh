@@ -41,19 +41,26 @@ __device__ __forceinline__ void cell_smooth64_at(int n, double* __restrict__ phi
     phi[id] = not_one(c.omega) ? fma(c.omega, v - old, old) : v;
     return;
   }
-  long long b[18];
-  gather_bits(phi + id, nbr(), b);
   const double sv = src[id];
   const double fv = f ? f[id] : 0.0;
   double face, M;
-  stencil_forms(phi + id, nbr, b, c.mode != OP_LINEAR, face, M);
   double acc = fma(fv, -c.h2_6, s_c);
-  if (c.mode == OP_SQRT) {
-    acc = fma(c.upd_s, sqrt_clamped_fix(fma(c.e1, M, sv)), acc);
+  if (c.mode == OP_LINEAR) {
+    long long b[6];
+    gather_bits(phi + id, nbr(), b);
+    stencil_forms(phi + id, nbr, b, false, face, M);
+    acc = fma(-c.h2_6, sv, acc);
   } else {
-    double q;
-    bool g;
-    acc = fma(-c.h2_6, root_of_M(M, sv, c, q, g), acc);
+    long long b[18];
+    gather_bits(phi + id, nbr(), b);
+    stencil_forms(phi + id, nbr, b, c.mode == OP_CONJ, face, M);
+    if (c.mode == OP_SQRT) {
+      acc = fma(c.upd_s, sqrt_clamped_fix(fma(c.e1, M, sv)), acc);
+    } else {
+      double q;
+      bool g;
+      acc = fma(-c.h2_6, root_of_M(M, sv, c, q, g), acc);
+    }
   }
   const double v = fma(face, 1.0 / 6.0, acc);
   if (not_one(c.omega))
@@ -102,10 +109,18 @@ __device__ __forceinline__ double cell_defect_fix64(const double* __restrict__ p
     const double D = root_Dc(s, phi[id], src, c, g);
     return fma((s.sx + s.sy + s.sz) - 6.0 * phi[id], c.inv_h2, -D);
   }
+  double lap, M;
+  if (c.mode == OP_LINEAR) {
+    long long b[7];
+    gather_bits(phi + id, nbr(), b);
+    stencil_forms(phi + id, nbr, b, false, lap, M);
+    q = 1.0;
+    g = false;
+    return fma(lap, c.inv_h2, -src);
+  }
   long long b[19];
   gather_bits(phi + id, nbr(), b);
-  double lap, M;
-  stencil_forms(phi + id, nbr, b, c.mode != OP_LINEAR, lap, M);
+  stencil_forms(phi + id, nbr, b, c.mode == OP_CONJ, lap, M);
   return fma(lap, c.inv_h2, -root_of_M(M, src, c, q, g));
 }
 

@@ -235,17 +235,19 @@ __device__ __forceinline__ double root_D(const StencilT<double>& s, double src,
   return (2.0 * u) / (1.0 + sqrt(q));
 }
 
-// The 18 neighbours of a cell (and the cell itself with NV = 19) as bit patterns, in
-// the order x, y, z face pairs, the xy, xz, yz cells as (++, --, +-, -+), the centre.
+// The 18 neighbours of a cell (with NV = 6 those across its faces alone; with NV = 7 and 19
+// the cell itself too) as bit patterns, in the order x, y, z face pairs, the xy, xz, yz cells
+// as (++, --, +-, -+), the centre.
 template <int NV>
 __device__ __forceinline__ void gather_bits(const double* __restrict__ c, const NbrOff& o,
                                             long long (&b)[NV]) {
-  const int off[19] = {o.xp,        o.xm,        o.yp,        o.ym,        o.zp,
-                       o.zm,        o.xp + o.yp, o.xm + o.ym, o.xp + o.ym, o.xm + o.yp,
-                       o.xp + o.zp, o.xm + o.zm, o.xp + o.zm, o.xm + o.zp, o.yp + o.zp,
-                       o.ym + o.zm, o.yp + o.zm, o.ym + o.zp, 0};
+  const int off[18] = {o.xp,        o.xm,        o.yp,        o.ym,        o.zp,        o.zm,
+                       o.xp + o.yp, o.xm + o.ym, o.xp + o.ym, o.xm + o.yp, o.xp + o.zp,
+                       o.xm + o.zm, o.xp + o.zm, o.xm + o.zp, o.yp + o.zp, o.ym + o.zm,
+                       o.yp + o.zm, o.ym + o.zp};
 #pragma unroll
-  for (int k = 0; k < NV; ++k) b[k] = __double_as_longlong(c[off[k]]);
+  for (int k = 0; k < NV; ++k)
+    b[k] = __double_as_longlong(c[(NV & 1) && k == NV - 1 ? 0 : off[k]]);
 }
 
 // stencil_forms of the cell at c in FP64, for values that fix_align refuses.  Not
@@ -255,41 +257,43 @@ static __device__ __noinline__ void stencil_forms_fp64(const double* c, NbrOff o
   const StencilT<double> s = gather_at(c, o);
   const double sum = s.sx + s.sy + s.sz;
   const double B = fma(s.cxy, s.cxy, fma(s.cxz, s.cxz, s.cyz * s.cyz));
-  *face = nv == 19 ? sum - 6.0 * *c : sum;
+  *face = (nv & 1) ? sum - 6.0 * *c : sum;
   *M = fma(0.375, B, 2.0 * half_A(s));
 }
 
 // What the operator needs of the stencil at `at` (b: its gather_bits, used up; nbr()
 // its offsets):
-//   face = Sx + Sy + Sz, with the centre (NV = 19) Sx + Sy + Sz - 6 phi;
-//   M = A + (3/8) B of Sigma_d h^4 = A/3 + B/8 (0 unless quad).
+//   face = Sx + Sy + Sz, with the centre (NV = 7, 19) Sx + Sy + Sz - 6 phi;
+//   M = A + (3/8) B of Sigma_d h^4 = A/3 + B/8 (0 with NV = 6, 7: the linear form).
+// near: of fix_align.
 template <int NV, typename Nbr>
 __device__ __forceinline__ void stencil_forms(const double* at, Nbr nbr, long long (&b)[NV],
-                                              bool quad, double& face, double& M) {
+                                              bool near, double& face, double& M) {
   FixRef r;
   M = 0.0;
-  if (!fix_align(b, r)) {
+  if (!fix_align(b, r, near)) {
     double fs, ms;
     stencil_forms_fp64(at, nbr(), NV, &fs, &ms);
     face = fs;
-    if (quad) M = ms;
+    if (NV >= 18) M = ms;
     return;
   }
   unsigned long long u[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) u[k] = (unsigned long long)b[k];
   const unsigned long long sx = u[0] + u[1], sy = u[2] + u[3], sz = u[4] + u[5];
-  const unsigned long long sub = NV == 19 ? 6 * u[NV - 1] : (unsigned long long)r.off6;
+  const unsigned long long sub = (NV & 1) ? 6 * u[NV - 1] : (unsigned long long)r.off6;
   face = fix_signed((long long)(sx + sy + sz - sub), r);
-  if (!quad) return;
-  const long long a[3] = {(long long)(sx - sy), (long long)(sx - sz), (long long)(sy - sz)};
-  const long long c[3] = {(long long)((u[6] + u[7]) - (u[8] + u[9])),
-                          (long long)((u[10] + u[11]) - (u[12] + u[13])),
-                          (long long)((u[14] + u[15]) - (u[16] + u[17]))};
-  int sh;
-  unsigned top;
-  const unsigned long long N = fix_quad(a, c, sh, top);
-  M = fix_double(N, 64 - 2 * sh + 2 * r.ue);
+  if constexpr (NV >= 18) {
+    const long long a[3] = {(long long)(sx - sy), (long long)(sx - sz), (long long)(sy - sz)};
+    const long long c[3] = {(long long)((u[6] + u[7]) - (u[8] + u[9])),
+                            (long long)((u[10] + u[11]) - (u[12] + u[13])),
+                            (long long)((u[14] + u[15]) - (u[16] + u[17]))};
+    int sh;
+    unsigned top;
+    const unsigned long long N = fix_quad(a, c, sh, top);
+    M = fix_double(N, 64 - 2 * sh + 2 * r.ue);
+  }
 }
 
 // sqrt_clamped with the square root of a normal q on the integer pipe.

@@ -135,11 +135,17 @@ constexpr int kFixMinExp = 640, kFixMaxExp = 1470;
 // Replace the bit patterns b[] by integers of one unit; false when the values have no
 // such form (b is then unchanged).
 //
-// NV = 18 leaves the largest below 2^60, for sums of six; NV = 19 (with the centre, of
-// which six are subtracted) below 2^59.
+// The first six are those across the cell's faces; NV = 18 adds the twelve across its edges;
+// NV = 7 and 19 have the centre last, of which six are subtracted.  Without a centre the
+// largest stays below 2^60, for sums of six, with one below 2^59.
+//
+// near: also false where values across the edges would cut off more of the others than FP64
+// does (the sums of those stand alone unless the squares of all enter beside them at the
+// weight of the square-root form).
 template <int NV>
-MG_HD bool fix_align(long long (&b)[NV], FixRef& r) {
-  constexpr int kUp = NV == 19 ? 6 : 7;  // bits above a significand
+MG_HD bool fix_align(long long (&b)[NV], FixRef& r, bool near = false) {
+  constexpr bool kCentre = NV == 7 || NV == 19;
+  constexpr int kUp = kCentre ? 6 : 7;  // bits above a significand
   const int h0 = fix_hi(b[0]);
   int diff = 0;
 #pragma unroll
@@ -173,12 +179,18 @@ MG_HD bool fix_align(long long (&b)[NV], FixRef& r) {
     }
   }
   int em = 0;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
+  auto largest = [&](int k) {
     const int e = fix_hi(b[k]) & 0x7ff00000;
     em = e > em ? e : em;
-  }
+  };
+#pragma unroll
+  for (int k = 0; k < 6; ++k) largest(k);
+  if (kCentre) largest(NV - 1);
+  const int ef = em;
+#pragma unroll
+  for (int k = 6; k < NV; ++k) largest(k);
   if (em < (kFixMinExp << 20) || em > (kFixMaxExp << 20)) return false;
+  if (near && em - ef > ((kUp - 2) << 20)) return false;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     const int h = fix_hi(b[k]);
