@@ -105,7 +105,9 @@ __global__ void __launch_bounds__(256) kb_smooth64(const BItem* __restrict__ ite
     pick(it.f != nullptr, it.op.mode == OP_LINEAR, run);
     return;
   }
-  b_smooth_colour64(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, blk);
+  by_mode(it.op.mode, [&](auto m) {
+    b_smooth_colour64<m()>(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, blk);
+  });
 }
 
 __global__ void __launch_bounds__(256) kb_residual_restrict64(const BItem* __restrict__ items,
@@ -124,8 +126,10 @@ __global__ void __launch_bounds__(256) kb_residual_restrict64(const BItem* __res
     if (threadIdx.x == 0) it.part[blk] = p;
     return;
   }
-  b_residual_restrict64(it.n, it.phi, it.src, it.f, it.op, it.cphi, it.cphihat, it.cf, it.part,
-                        blk);
+  by_mode(it.op.mode, [&](auto m) {
+    b_residual_restrict64<m()>(it.n, it.phi, it.src, it.f, it.op, it.cphi, it.cphihat, it.cf,
+                               it.part, blk);
+  });
 }
 
 // One block per item.  mode 0: partials of a residual-restriction (one per 256
@@ -165,7 +169,9 @@ __global__ void __launch_bounds__(256) kb_fas_rhs64(const BItem* __restrict__ it
                               o.z, S);
     return;
   }
-  b_fas_rhs64(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, blk);
+  by_mode(it.cop.mode, [&](auto m) {
+    b_fas_rhs64<m()>(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, blk);
+  });
 }
 
 __global__ void __launch_bounds__(256) kb_prolong64(const BItem* __restrict__ items, int count) {
@@ -200,7 +206,9 @@ __global__ void __launch_bounds__(256) kb_handoff64(const BItem* __restrict__ it
     if (threadIdx.x == 0) it.part[blk] = p;
     return;
   }
-  b_residual_handoff64(it.n, it.phi, it.src, it.op, it.sc, out, it.part, blk);
+  by_mode(it.op.mode, [&](auto m) {
+    b_residual_handoff64<m()>(it.n, it.phi, it.src, it.op, it.sc, out, it.part, blk);
+  });
 }
 
 __global__ void __launch_bounds__(256) kb_update64(const BItem* __restrict__ items, int count) {

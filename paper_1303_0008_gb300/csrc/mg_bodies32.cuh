@@ -114,6 +114,7 @@ struct Handoff {
   }
 };
 
+template <int MODE>
 __device__ __forceinline__ void b_residual_handoff64(int n, const double* __restrict__ phi,
                                                      const double* __restrict__ src,
                                                      const OpConst64& c,
@@ -133,7 +134,7 @@ __device__ __forceinline__ void b_residual_handoff64(int n, const double* __rest
     split3((unsigned)t, n, i, j, k);
     double q;
     bool guard;
-    const double d = cell_defect_fix64(phi, n, i, j, k, t, src[t], c, q, guard);
+    const double d = cell_defect_fix64<MODE>(phi, n, i, j, k, t, src[t], c, q, guard);
     partial_add(p, d, guard);
     out.store(n, i, j, k, t, phi[t], lam - d, q);
   }

@@ -28,13 +28,14 @@ static __device__ __noinline__ void relax64(double* phi, double v, double omega)
 //   phi_new = (Sx + Sy + Sz - h^2 (D + f + lambda)) / 6.
 // In the sqrt form, D = k2s sqrt(q) - k2, so phi_new = upd_s sqrt(q) + (Sx+Sy+Sz)/6 -
 // h^2 f/6 + C with the block-wide C = -h^2 (lambda - k2)/6 (s_c).
+template <int MODE>
 __device__ __forceinline__ void cell_smooth64_at(int n, double* __restrict__ phi,
                                                  const double* __restrict__ src,
                                                  const double* __restrict__ f, double s_c,
                                                  const OpConst64& c, int i, int j, int k) {
   const long long id = lidx(i, j, k, n);
   auto nbr = [&] { return nbr_offsets(i, j, k, n); };
-  if (c.mode == OP_GENW) {
+  if constexpr (MODE == OP_GENW) {
     const double old = phi[id];
     const double v = genw_newton(gather_at(phi + id, nbr()), old, src[id],
                                  (f ? f[id] : 0.0) + s_c, c);
@@ -45,7 +46,7 @@ __device__ __forceinline__ void cell_smooth64_at(int n, double* __restrict__ phi
   const double fv = f ? f[id] : 0.0;
   double face, M;
   double acc = fma(fv, -c.h2_6, s_c);
-  if (c.mode == OP_LINEAR) {
+  if constexpr (MODE == OP_LINEAR) {
     long long b[6];
     gather_bits(phi + id, nbr(), b);
     stencil_forms(phi + id, nbr, b, false, face, M);
@@ -53,13 +54,13 @@ __device__ __forceinline__ void cell_smooth64_at(int n, double* __restrict__ phi
   } else {
     long long b[18];
     gather_bits(phi + id, nbr(), b);
-    stencil_forms(phi + id, nbr, b, c.mode == OP_CONJ, face, M);
-    if (c.mode == OP_SQRT) {
+    stencil_forms(phi + id, nbr, b, MODE == OP_CONJ, face, M);
+    if constexpr (MODE == OP_SQRT) {
       acc = fma(c.upd_s, sqrt_clamped_fix(fma(c.e1, M, sv)), acc);
     } else {
       double q;
       bool g;
-      acc = fma(-c.h2_6, root_of_M(M, sv, c, q, g), acc);
+      acc = fma(-c.h2_6, root_of_M<MODE>(M, sv, c, q, g), acc);
     }
   }
   const double v = fma(face, 1.0 / 6.0, acc);
@@ -71,6 +72,7 @@ __device__ __forceinline__ void cell_smooth64_at(int n, double* __restrict__ phi
 
 // One cell of a colour stage: t indexes the colour's n^3/4 cells; t >= n^3/4 does
 // nothing.
+template <int MODE>
 __device__ __forceinline__ void cell_smooth64(int n, double* __restrict__ phi,
                                               const double* __restrict__ src,
                                               const double* __restrict__ f, double s_c,
@@ -82,9 +84,10 @@ __device__ __forceinline__ void cell_smooth64(int n, double* __restrict__ phi,
   split3((unsigned)t, hn, m, jj, k);
   const int i = 2 * m + ((colour ^ k) & 1);
   const int j = 2 * jj + (((colour >> 1) ^ k) & 1);
-  cell_smooth64_at(n, phi, src, f, s_c, c, i, j, k);
+  cell_smooth64_at<MODE>(n, phi, src, f, s_c, c, i, j, k);
 }
 
+template <int MODE>
 __device__ __forceinline__ void b_smooth_colour64(int n, double* __restrict__ phi,
                                                          const double* __restrict__ src,
                                                          const double* __restrict__ f,
@@ -94,23 +97,24 @@ __device__ __forceinline__ void b_smooth_colour64(int n, double* __restrict__ ph
   __shared__ double s_c;
   if (threadIdx.x == 0) s_c = smooth_scalar64(sc, c);
   __syncthreads();
-  cell_smooth64(n, phi, src, f, s_c, c, colour, (long long)blk * blockDim.x + threadIdx.x);
+  cell_smooth64<MODE>(n, phi, src, f, s_c, c, colour, (long long)blk * blockDim.x + threadIdx.x);
 }
 
 // The defect L(phi) of cell (i,j,k) (linear index id) without a right-hand side, its
 // discriminant (1 where the mode has none) and guard flag.
+template <int MODE>
 __device__ __forceinline__ double cell_defect_fix64(const double* __restrict__ phi, int n, int i,
                                                     int j, int k, long long id, double src,
                                                     const OpConst64& c, double& q, bool& g) {
   auto nbr = [&] { return nbr_offsets(i, j, k, n); };
-  if (c.mode == OP_GENW) {
+  if constexpr (MODE == OP_GENW) {
     const StencilT<double> s = gather_at(phi + id, nbr());
     q = 1.0;
     const double D = root_Dc(s, phi[id], src, c, g);
     return fma((s.sx + s.sy + s.sz) - 6.0 * phi[id], c.inv_h2, -D);
   }
   double lap, M;
-  if (c.mode == OP_LINEAR) {
+  if constexpr (MODE == OP_LINEAR) {
     long long b[7];
     gather_bits(phi + id, nbr(), b);
     stencil_forms(phi + id, nbr, b, false, lap, M);
@@ -120,11 +124,12 @@ __device__ __forceinline__ double cell_defect_fix64(const double* __restrict__ p
   }
   long long b[19];
   gather_bits(phi + id, nbr(), b);
-  stencil_forms(phi + id, nbr, b, c.mode == OP_CONJ, lap, M);
-  return fma(lap, c.inv_h2, -root_of_M(M, src, c, q, g));
+  stencil_forms(phi + id, nbr, b, MODE == OP_CONJ, lap, M);
+  return fma(lap, c.inv_h2, -root_of_M<MODE>(M, src, c, q, g));
 }
 
 // The defect d = L(phi) - f of fine cell (i,j,k) and its guard flag; ctr returns phi there.
+template <int MODE>
 __device__ __forceinline__ double fine_defect64(int nf, const double* __restrict__ phi,
                                                const double* __restrict__ src,
                                                const double* __restrict__ f,
@@ -132,10 +137,11 @@ __device__ __forceinline__ double fine_defect64(int nf, const double* __restrict
                                                long long id, double& ctr, bool& g) {
   ctr = phi[id];
   double q;
-  const double d = cell_defect_fix64(phi, nf, i, j, k, id, src[id], c, q, g);
+  const double d = cell_defect_fix64<MODE>(phi, nf, i, j, k, id, src[id], c, q, g);
   return f ? d - f[id] : d;
 }
 
+template <int MODE>
 __device__ __forceinline__ void b_residual_restrict64(
     int nf, const double* __restrict__ phi, const double* __restrict__ src,
     const double* __restrict__ f, OpConst64 c, double* __restrict__ phi_c,
@@ -163,7 +169,7 @@ __device__ __forceinline__ void b_residual_restrict64(
       const long long id = lidx(i, j, k, nf);
       bool g;
       double ctr;
-      const double d = fine_defect64(nf, phi, src, f, c, i, j, k, id, ctr, g);
+      const double d = fine_defect64<MODE>(nf, phi, src, f, c, i, j, k, id, ctr, g);
       const bool fin = finite_bits(d);
       const long long key = order_key(d);
       kmax = (fin && key > kmax) ? key : kmax;
@@ -184,7 +190,7 @@ __device__ __forceinline__ void b_residual_restrict64(
         const int i = 2 * I + (ch & 1), j = 2 * J + ((ch >> 1) & 1), k = 2 * K + (ch >> 2);
         bool g;
         double ctr;
-        partial_add(p, fine_defect64(nf, phi, src, f, c, i, j, k, lidx(i, j, k, nf), ctr, g), g);
+        partial_add(p, fine_defect64<MODE>(nf, phi, src, f, c, i, j, k, lidx(i, j, k, nf), ctr, g), g);
       }
     }
     phi_c[t] = sphi * 0.125;
@@ -200,6 +206,7 @@ __device__ __forceinline__ void b_residual_restrict64(
 // and guard flag (t indexes the nf^3 fine cells), then b_restrict_defects64
 // walks every coarse cell's 8 children in the order of b_residual_restrict64,
 // with its block partition, so both give the same bits.
+template <int MODE>
 __device__ __forceinline__ void cell_defect64(int nf, const double* __restrict__ phi,
                                               const double* __restrict__ src,
                                               const double* __restrict__ f, const OpConst64& c,
@@ -211,7 +218,7 @@ __device__ __forceinline__ void cell_defect64(int nf, const double* __restrict__
   split3((unsigned)t, nf, i, j, k);
   bool g;
   double ctr;
-  dout[t] = fine_defect64(nf, phi, src, f, c, i, j, k, t, ctr, g);
+  dout[t] = fine_defect64<MODE>(nf, phi, src, f, c, i, j, k, t, ctr, g);
   gout[t] = g ? 1 : 0;
 }
 
@@ -282,6 +289,7 @@ __device__ __forceinline__ void b_finalize(const Partial* __restrict__ partials,
 // One coarse cell of the FAS right-hand side f_c = L_c(phi_c) - f_c + lambda_f
 // (t indexes the nc^3 cells; lam_f is the fine level's lambda; cell 0 also clears
 // the coarse lambda).
+template <int MODE>
 __device__ __forceinline__ void cell_fas_rhs64(int nc, const double* __restrict__ phi_c,
                                                const double* __restrict__ src_c,
                                                double* __restrict__ f_c, const OpConst64& c,
@@ -294,17 +302,18 @@ __device__ __forceinline__ void cell_fas_rhs64(int nc, const double* __restrict_
   split3((unsigned)t, nc, i, j, k);
   double q;
   bool g;
-  const double L = cell_defect_fix64(phi_c, nc, i, j, k, t, src_c[t], c, q, g);
+  const double L = cell_defect_fix64<MODE>(phi_c, nc, i, j, k, t, src_c[t], c, q, g);
   f_c[t] = L - f_c[t] + lam_f;
 }
 
+template <int MODE>
 __device__ __forceinline__ void b_fas_rhs64(int nc, const double* __restrict__ phi_c,
                                                    const double* __restrict__ src_c,
                                                    double* __restrict__ f_c, OpConst64 c,
                                                    const LevelScalars* __restrict__ fine_sc,
                                                    LevelScalars* __restrict__ coarse_sc,
     long long blk) {
-  cell_fas_rhs64(nc, phi_c, src_c, f_c, c, fine_sc->lambda, coarse_sc,
+  cell_fas_rhs64<MODE>(nc, phi_c, src_c, f_c, c, fine_sc->lambda, coarse_sc,
                  (long long)blk * blockDim.x + threadIdx.x);
 }
 

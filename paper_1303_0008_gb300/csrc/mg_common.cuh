@@ -19,6 +19,7 @@
 
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <type_traits>
 
 #include "mg_fix64.cuh"
 
@@ -31,6 +32,18 @@ enum OpMode : int {
   OP_CONJ = 2,    // physical root as 2u/(1+sqrt(q)) for small |alpha|; src = kappa delta
   OP_GENW = 3     // splitting w != 1/3: Sigma involves the centre value (full Newton step)
 };
+
+// run(mode) with the mode as a type: the kernels that go cell by cell are compiled for one
+// mode each, without the others' code and registers.
+template <typename Run>
+__host__ __device__ __forceinline__ void by_mode(int mode, Run run) {
+  switch (mode) {
+    case OP_LINEAR: run(std::integral_constant<int, OP_LINEAR>{}); break;
+    case OP_SQRT: run(std::integral_constant<int, OP_SQRT>{}); break;
+    case OP_CONJ: run(std::integral_constant<int, OP_CONJ>{}); break;
+    default: run(std::integral_constant<int, OP_GENW>{});
+  }
+}
 
 // Per-level constants of the FP64 operator.
 struct OpConst64 {
@@ -305,12 +318,13 @@ __device__ __forceinline__ double sqrt_clamped_fix(double q) {
 
 // The root D of Eq. two_branch from M (stencil_forms) and the source term; q is the
 // discriminant (1 in the linear mode) and guard whether it is negative.
+template <int MODE>
 __device__ __forceinline__ double root_of_M(double M, double src, const OpConst64& c, double& q,
                                             bool& guard) {
   q = 1.0;
   guard = false;
-  if (c.mode == OP_LINEAR) return src;
-  if (c.mode == OP_SQRT) {
+  if (MODE == OP_LINEAR) return src;
+  if (MODE == OP_SQRT) {
     q = fma(c.e1, M, src);
     guard = neg_guard(q);
     return fma(c.k2s, sqrt_clamped_fix(q), -c.k2);

@@ -24,7 +24,11 @@ namespace mg {
 // ---------------------------------------------------------------------------
 // A warp takes a block of 8 x 2 x 2 of the colour's cells (x, y, z), a CTA warps / 2 of
 // them along x on each of two pairs of planes: a compact block mostly lies in one binade
-// of the field, which is the cheapest path of fix_align.
+// of the field, which is the cheapest path of fix_align.  One kernel per mode (by_mode), here
+// and below: with all of them in one, the linear and the general form (40 and 32 registers)
+// carried the integer form's 80, and its code ran longer by the others' branches (FP64 solves
+// of 32^3 2.86 -> 2.73 ms, 64^3 4.60 -> 4.37, 128^3 8.31 -> 8.04).
+template <int MODE>
 __global__ void __launch_bounds__(256) k_smooth_colour64(int n, double* __restrict__ phi,
                                                          const double* __restrict__ src,
                                                          const double* __restrict__ f,
@@ -40,7 +44,7 @@ __global__ void __launch_bounds__(256) k_smooth_colour64(int n, double* __restri
   const int jj = (int)blockIdx.y * 2 + ((lane >> 3) & 1);
   const int k = (int)blockIdx.z * 4 + (w & 1) * 2 + (lane >> 4);
   if (m >= hn || jj >= hn || k >= n) return;
-  cell_smooth64_at(n, phi, src, f, s_c, c, 2 * m + ((colour ^ k) & 1),
+  cell_smooth64_at<MODE>(n, phi, src, f, s_c, c, 2 * m + ((colour ^ k) & 1),
                    2 * jj + (((colour >> 1) ^ k) & 1), k);
 }
 
@@ -58,6 +62,7 @@ __global__ void __launch_bounds__(256, 4) k_smooth_tile64(int n, double* __restr
 }
 
 // d = L^h phi - f with block partial norms.
+template <int MODE>
 __global__ void __launch_bounds__(256) k_residual64(int n, const double* __restrict__ phi,
                                                     const double* __restrict__ src,
                                                     const double* __restrict__ f,
@@ -73,7 +78,7 @@ __global__ void __launch_bounds__(256) k_residual64(int n, const double* __restr
     split3((unsigned)t, n, i, j, k);
     bool g;
     double ctr;
-    const double d = fine_defect64(n, phi, src, f, c, i, j, k, t, ctr, g);
+    const double d = fine_defect64<MODE>(n, phi, src, f, c, i, j, k, t, ctr, g);
     if (dout) dout[t] = d;
     partial_add(p, d, g);
   }
@@ -107,12 +112,13 @@ __global__ void __launch_bounds__(256, 4) k_residual_tile64(int n, const double*
 
 // Residual of the 8 children of each coarse cell, averaged (full weighting),
 // together with R phi; the partial norms cover every fine cell.
+template <int MODE>
 __global__ void __launch_bounds__(256) k_residual_restrict64(
     int nf, const double* __restrict__ phi, const double* __restrict__ src,
     const double* __restrict__ f, OpConst64 c, double* __restrict__ phi_c,
     double* __restrict__ phihat_c, double* __restrict__ rd_c, Partial* __restrict__ partials) {
   PdlScope pdl_scope;
-  b_residual_restrict64(nf, phi, src, f, c, phi_c, phihat_c, rd_c, partials, blockIdx.x);
+  b_residual_restrict64<MODE>(nf, phi, src, f, c, phi_c, phihat_c, rd_c, partials, blockIdx.x);
 }
 
 // The same for levels of many tiles, one partial per tile.
@@ -134,13 +140,14 @@ __global__ void __launch_bounds__(256, 2) k_residual_restrict_tile64(
 // fill only a few 256-thread blocks: per fine cell the defect and guard flag
 // (blocks of any size), then the walk over each coarse cell's children in the
 // order and 256-thread partition of k_residual_restrict64 (the same bits).
+template <int MODE>
 __global__ void __launch_bounds__(256) k_defect64(int nf, const double* __restrict__ phi,
                                                   const double* __restrict__ src,
                                                   const double* __restrict__ f, OpConst64 c,
                                                   double* __restrict__ dout,
                                                   unsigned char* __restrict__ gout) {
   PdlScope pdl_scope;
-  cell_defect64(nf, phi, src, f, c, dout, gout, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+  cell_defect64<MODE>(nf, phi, src, f, c, dout, gout, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 __global__ void __launch_bounds__(256) k_restrict_defects64(
@@ -170,13 +177,14 @@ __global__ void __launch_bounds__(1024) k_finalize(const Partial* __restrict__ p
 }
 
 // f^H = L^H(R phi) - (R d - lambda^h); lambda^H starts at 0.
+template <int MODE>
 __global__ void __launch_bounds__(256) k_fas_rhs64(int nc, const double* __restrict__ phi_c,
                                                    const double* __restrict__ src_c,
                                                    double* __restrict__ f_c, OpConst64 c,
                                                    const LevelScalars* __restrict__ fine_sc,
                                                    LevelScalars* __restrict__ coarse_sc) {
   PdlScope pdl_scope;
-  b_fas_rhs64(nc, phi_c, src_c, f_c, c, fine_sc, coarse_sc, blockIdx.x);
+  b_fas_rhs64<MODE>(nc, phi_c, src_c, f_c, c, fine_sc, coarse_sc, blockIdx.x);
 }
 
 // The same for levels of many tiles.
@@ -368,7 +376,11 @@ void launch_finalize(cudaStream_t st, const Partial* partials, int nparts, doubl
 void launch_smooth64(cudaStream_t st, int n, double* phi, const double* src, const double* f,
                      const LevelScalars* sc, const OpConst64& c, int sweeps, EventPairs* timer) {
   const int hn = n / 2;
-  const unsigned tpb = (unsigned)tpb_for((long long)hn * hn * n);
+  // A splitting constant of its own runs in FP64 with 32 registers, all CTAs at once: wide ones
+  // that reach past the row leave some SMs idle warps only (96^3 solves 11.3 against 9.6 ms).
+  const unsigned tpb = c.mode == OP_GENW && hn % 32 != 0
+                           ? 64u
+                           : (unsigned)tpb_for((long long)hn * hn * n);
   const unsigned bx = tpb / 8;  // cells of the colour along x per CTA
   const dim3 grid((hn + bx - 1) / bx, (hn + 1) / 2, (n + 3) / 4);
   const bool tiles = smooth_in_tiles(n, c), lin = c.mode == OP_LINEAR;
@@ -383,7 +395,9 @@ void launch_smooth64(cudaStream_t st, int n, double* phi, const double* src, con
       if (tiles)
         launch_k(tile_kernel, tile_grid(n), 256, 0, st, n, phi, src, f, sc, c, colour);
       else
-        launch_k(k_smooth_colour64, grid, tpb, 0, st, n, phi, src, f, sc, c, colour);
+        by_mode(c.mode, [&](auto m) {
+          launch_k(k_smooth_colour64<m()>, grid, tpb, 0, st, n, phi, src, f, sc, c, colour);
+        });
       if (timed) timer->end(st);
     }
   count_launches(4LL * sweeps);
@@ -398,9 +412,12 @@ void launch_residual64(cudaStream_t st, int n, const double* phi, const double* 
   const bool tiles = in_tiles(n, c);
   const unsigned nb = tiles ? tile_count(n) : blocks_for(cells, 256);
   if (tiles)
-    launch_k(c.mode == OP_LINEAR ? k_residual_tile64<true> : k_residual_tile64<false>, tile_grid(n), 256, 0, st, n, phi, src, f, dout, c, partials);
+    launch_k(c.mode == OP_LINEAR ? k_residual_tile64<true> : k_residual_tile64<false>,
+             tile_grid(n), 256, 0, st, n, phi, src, f, dout, c, partials);
   else
-    launch_k(k_residual64, nb, 256, 0, st, n, phi, src, f, dout, c, partials);
+    by_mode(c.mode, [&](auto m) {
+      launch_k(k_residual64<m()>, nb, 256, 0, st, n, phi, src, f, dout, c, partials);
+    });
   launch_finalize(st, partials, (int)nb, (double)cells, periodic, sc);
   count_launches(1);
 }
@@ -422,13 +439,18 @@ void launch_residual_restrict64(cudaStream_t st, int nf, const double* phi, cons
              tile_grid(nf), 256, 0, st, nf, phi, src, f, c, phi_c, phihat_c, rd_c, partials);
   } else if (def && guard && fcells <= kTwoStepMaxFine) {
     const int tpb = tpb_for(fcells);
-    launch_k(k_defect64, blocks_for(fcells, tpb), tpb, 0, st, nf, phi, src, f, c, def, guard);
+    by_mode(c.mode, [&](auto m) {
+      launch_k(k_defect64<m()>, blocks_for(fcells, tpb), tpb, 0, st, nf, phi, src, f, c, def,
+               guard);
+    });
     launch_k(k_restrict_defects64, nb, 256, 0, st, nf, phi, (const double*)def,
              (const unsigned char*)guard, phi_c, phihat_c, rd_c, partials);
     count_launches(1);
   } else {
-    launch_k(k_residual_restrict64, nb, 256, 0, st, nf, phi, src, f, c, phi_c, phihat_c, rd_c,
-             partials);
+    by_mode(c.mode, [&](auto m) {
+      launch_k(k_residual_restrict64<m()>, nb, 256, 0, st, nf, phi, src, f, c, phi_c, phihat_c,
+               rd_c, partials);
+    });
   }
   launch_finalize(st, partials, (int)nb, (double)fcells, 1, sc);
   count_launches(1);
@@ -440,11 +462,13 @@ void launch_fas_rhs64(cudaStream_t st, int nc, const double* phi_c, const double
   const long long cells = (long long)nc * nc * nc;
   const int tpb = tpb_for(cells);
   if (in_tiles(nc, c))
-    launch_k(c.mode == OP_LINEAR ? k_fas_rhs_tile64<true> : k_fas_rhs_tile64<false>, tile_grid(nc), 256, 0, st, nc, phi_c, src_c, f_c, c, fine_sc,
-             coarse_sc);
+    launch_k(c.mode == OP_LINEAR ? k_fas_rhs_tile64<true> : k_fas_rhs_tile64<false>,
+             tile_grid(nc), 256, 0, st, nc, phi_c, src_c, f_c, c, fine_sc, coarse_sc);
   else
-    launch_k(k_fas_rhs64, blocks_for(cells, tpb), tpb, 0, st, nc, phi_c, src_c, f_c, c, fine_sc,
-             coarse_sc);
+    by_mode(c.mode, [&](auto m) {
+      launch_k(k_fas_rhs64<m()>, blocks_for(cells, tpb), tpb, 0, st, nc, phi_c, src_c, f_c, c,
+               fine_sc, coarse_sc);
+    });
   count_launches(1);
 }
 

@@ -39,6 +39,7 @@ namespace mg {
 // ---------------------------------------------------------------------------
 // FP64 outer residual with the FP32 hand-off.
 // ---------------------------------------------------------------------------
+template <int MODE>
 __global__ void __launch_bounds__(256) k_residual_handoff64(int n, const double* __restrict__ phi,
                                                             const double* __restrict__ src,
                                                             OpConst64 c,
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(256) k_residual_handoff64(int n, const double*
                                                             Handoff out,
                                                             Partial* __restrict__ partials) {
   PdlScope pdl_scope;
-  b_residual_handoff64(n, phi, src, c, sc, out, partials, blockIdx.x);
+  b_residual_handoff64<MODE>(n, phi, src, c, sc, out, partials, blockIdx.x);
 }
 
 // The same for levels of many tiles, one partial per tile.
@@ -588,11 +589,13 @@ struct CycleMixed {
     const unsigned nb = tiles ? tile_count(L.n) : nblk(L.cells, 256 * kHandoffCells);
     const Handoff out{L.rhs, L.q0, L.phi0, L.e, L.rhsc, L.q0c};
     if (tiles)
-      launch_k(ops[0].mode == OP_LINEAR ? k_handoff_tile64<true> : k_handoff_tile64<false>, tile_grid(L.n), 256, 0, st, L.n, L.phi, L.src, ops[0], d->d_sc,
-               out, d->d_part);
+      launch_k(ops[0].mode == OP_LINEAR ? k_handoff_tile64<true> : k_handoff_tile64<false>,
+               tile_grid(L.n), 256, 0, st, L.n, L.phi, L.src, ops[0], d->d_sc, out, d->d_part);
     else
-      launch_k(k_residual_handoff64, nb, 256, 0, st, L.n, L.phi, L.src, ops[0], d->d_sc, out,
-               d->d_part);
+      by_mode(ops[0].mode, [&](auto m) {
+        launch_k(k_residual_handoff64<m()>, nb, 256, 0, st, L.n, L.phi, L.src, ops[0], d->d_sc,
+                 out, d->d_part);
+      });
     count_launches(1);
     launch_finalize(st, d->d_part, (int)nb, (double)L.cells, 1, d->d_sc);
     cudaMemcpyAsync(d->h_sc, d->d_sc, sizeof(LevelScalars), cudaMemcpyDeviceToHost, st);

@@ -42,6 +42,7 @@ static __device__ __align__(256) NoAllocScratch g_noalloc_scratch;
 
 // d = L^h phi - f with the source term a*delta + b formed per cell (the same
 // fma as the source-preparation kernel, so the values match bit for bit).
+template <int MODE>
 __global__ void __launch_bounds__(kNoAllocThreads) k_residual64_noalloc(
     int n, const double* __restrict__ phi, const double* __restrict__ delta, double a, double b,
     const double* __restrict__ f, double* __restrict__ dout, OpConst64 c,
@@ -55,7 +56,7 @@ __global__ void __launch_bounds__(kNoAllocThreads) k_residual64_noalloc(
     split3((unsigned)t, n, i, j, k);
     double q;
     bool g;
-    double d = cell_defect_fix64(phi, n, i, j, k, t, fma(a, delta[t], b), c, q, g);
+    double d = cell_defect_fix64<MODE>(phi, n, i, j, k, t, fma(a, delta[t], b), c, q, g);
     if (f) d -= f[t];
     if (dout) dout[t] = d;
     partial_add(p, d, g);
@@ -156,7 +157,10 @@ extern "C" mg_status mg_op_residual_noalloc(int n, const double* phi, const doub
     (c.mode == OP_LINEAR ? k_residual_tile64_noalloc<true> : k_residual_tile64_noalloc<false>)
         <<<tile_grid(n), 256, 0, s>>>(n, phi, delta, a, b, f, d, c, scratch);
   else
-    k_residual64_noalloc<<<nb, kNoAllocThreads, 0, s>>>(n, phi, delta, a, b, f, d, c, scratch);
+    by_mode(c.mode, [&](auto m) {
+      k_residual64_noalloc<m()>
+          <<<nb, kNoAllocThreads, 0, s>>>(n, phi, delta, a, b, f, d, c, scratch);
+    });
   count_launches(1);
   launch_finalize(s, scratch->partials, (int)nb, (double)cells, 1, &scratch->scalars);
   cudaError_t e = cudaGetLastError();

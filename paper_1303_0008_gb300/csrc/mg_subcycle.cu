@@ -54,6 +54,7 @@ struct Phases {
   }
 };
 
+template <int MODE>
 __global__ void __launch_bounds__(256) k_subcycle64(const __grid_constant__ SubCycleArgs a) {
   PdlScope pdl_scope;
   __shared__ double s_c, s_lam;
@@ -68,7 +69,7 @@ __global__ void __launch_bounds__(256) k_subcycle64(const __grid_constant__ SubC
     for (int s = 0; s < sweeps; ++s)
       for (int colour = 0; colour < 4; ++colour)
         ph.spread(per, [&](long long t) {
-          cell_smooth64(L.n, L.phi, L.src, L.f, sc, L.op, colour, t);
+          cell_smooth64<MODE>(L.n, L.phi, L.src, L.f, sc, L.op, colour, t);
         });
   };
   for (int l = 0; l + 1 < a.nlev; ++l) {
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(256) k_subcycle64(const __grid_constant__ SubC
     const long long cc = (long long)C.n * C.n * C.n;
     smooth(L, a.nu_pre);
     ph.spread(8 * cc, [&](long long t) {
-      cell_defect64(L.n, L.phi, L.src, L.f, L.op, a.def64, a.guard, t);
+      cell_defect64<MODE>(L.n, L.phi, L.src, L.f, L.op, a.def64, a.guard, t);
     });
     const long long rr = nblk256(cc);
     ph.blocks(rr, [&](long long b) {
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(256) k_subcycle64(const __grid_constant__ SubC
     }
     const double lam = s_lam;
     ph.spread(cc, [&](long long t) {
-      cell_fas_rhs64(C.n, C.phi, C.src, C.f, C.op, lam, C.sc, t);
+      cell_fas_rhs64<MODE>(C.n, C.phi, C.src, C.f, C.op, lam, C.sc, t);
     });
   }
   {
@@ -208,19 +209,24 @@ void init_subcycle() {
   static bool done = false;
   if (done) return;
   done = true;
-  cudaFuncSetAttribute(k_subcycle64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       4 * sizeof(double) * 4096);
+  for (int mode : {OP_LINEAR, OP_SQRT, OP_CONJ, OP_GENW})
+    by_mode(mode, [](auto m) {
+      cudaFuncSetAttribute(k_subcycle64<m()>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           4 * sizeof(double) * 4096);
+      cudaFuncSetAttribute(k_subcycle64<m()>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    });
   cudaFuncSetAttribute(k_subcycle32, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        4 * sizeof(double) * 4096);
-  cudaFuncSetAttribute(k_subcycle64, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   cudaFuncSetAttribute(k_subcycle32, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   cudaGetLastError();
 }
 
 void launch_subcycle64(cudaStream_t st, const SubCycleArgs& a) {
   const int nc = a.lv[a.nlev - 1].n;
-  launch_cluster(k_subcycle64, st, a, 3 * sizeof(double) * (size_t)nc * nc * nc,
-                 kClusterCtas64);
+  by_mode(a.lv[0].op.mode, [&](auto m) {
+    launch_cluster(k_subcycle64<m()>, st, a, 3 * sizeof(double) * (size_t)nc * nc * nc,
+                   kClusterCtas64);
+  });
 }
 
 void launch_subcycle32(cudaStream_t st, const SubCycleArgs& a) {

@@ -305,7 +305,7 @@ __device__ __forceinline__ void b_smooth_tile64(int n, double* __restrict__ phi,
 #pragma unroll 1
   for (int s = 0; rare != 0; ++s, rare >>= 1) {
     const int k = k0 + 2 * s;
-    if ((rare & 1) && k < n) cell_smooth64_at(n, phi, src, f, s_c, c, i, j, k);
+    if ((rare & 1) && k < n) cell_smooth64_at<LIN ? OP_LINEAR : OP_SQRT>(n, phi, src, f, s_c, c, i, j, k);
   }
 }
 
@@ -469,9 +469,9 @@ __device__ __forceinline__ void tile_defects(int n, const double* __restrict__ p
     double qd, d;
     bool g;
     if (ok == 2)
-      d = fma(0.0, c.inv_h2, -root_of_M(0.0, src(id), c, qd, g));
+      d = fma(0.0, c.inv_h2, -root_of_M<LIN ? OP_LINEAR : OP_SQRT>(0.0, src(id), c, qd, g));
     else
-      d = cell_defect_fix64(phi, n, i, j, k, id, src(id), c, qd, g);
+      d = cell_defect_fix64<LIN ? OP_LINEAR : OP_SQRT>(phi, n, i, j, k, id, src(id), c, qd, g);
     cell(id, i, j, k, d, qd, g);
   }
 }
@@ -492,11 +492,12 @@ __device__ __forceinline__ Partial tile_reduce(Partial p, TileShared& S) {
   return p;
 }
 
+template <bool LIN>
 static __device__ __noinline__ double tile_defect_rare(const double* phi, int n, int i, int j,
                                                        int k, double src, const OpConst64* c,
                                                        bool* g) {
   double q;
-  return cell_defect_fix64(phi, n, i, j, k, lidx(i, j, k, n), src, *c, q, *g);
+  return cell_defect_fix64<LIN ? OP_LINEAR : OP_SQRT>(phi, n, i, j, k, lidx(i, j, k, n), src, *c, q, *g);
 }
 
 // Residual restriction of a tile (b_residual_restrict64).  A thread takes a column of 2 x 1
@@ -545,7 +546,7 @@ __device__ __forceinline__ Partial b_residual_restrict_tile64(
           mid[y] = up;
           q[y] += kTilePlane;
         }
-        if (!good) d = tile_defect_rare(phi, nf, i, j, k, src[id], &c, &g);
+        if (!good) d = tile_defect_rare<LIN>(phi, nf, i, j, k, src[id], &c, &g);
         if (F) d -= f[id];
         const bool fin = finite_bits(d);
         const long long key = order_key(d);
