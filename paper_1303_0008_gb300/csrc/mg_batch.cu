@@ -90,46 +90,57 @@ __device__ __forceinline__ void pick(bool f, bool lin, Run run) {
     f ? run(T{}, N{}) : run(N{}, N{});
 }
 
+// Each FP64 stage has a kernel for the levels that run in tiles and one for those that go cell
+// by cell, with a list each: in one kernel the small levels carried the tile's registers and
+// its 49 KB, and the large ones had one or two CTAs per SM where the single grids' kernels have
+// four.  (FP64 batches of 32^3 boxes took 1.15 to 1.2 times as long.)
 // ---- FP64 stages ----
-__global__ void __launch_bounds__(256) kb_smooth64(const BItem* __restrict__ items, int count,
-                                                   int colour) {
+__global__ void __launch_bounds__(256, 3) kb_smooth64(const BItem* __restrict__ items, int count,
+                                                      int colour) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
-  __shared__ TileShared S;
-  if (smooth_in_tiles(it.n, it.op)) {
-    const int3 o = tile_origin(it.n, blk);
-    auto run = [&](auto f, auto lin) {
-      b_smooth_tile64<decltype(f)::value, decltype(lin)::value>(
-          it.n, it.phi, it.src, it.f, it.sc, it.op, colour, o.x, o.y, o.z, S);
-    };
-    pick(it.f != nullptr, it.op.mode == OP_LINEAR, run);
-    return;
-  }
+  __shared__ double s_c;
+  if (threadIdx.x == 0) s_c = smooth_scalar64(it.sc, it.op);
+  __syncthreads();
   by_mode(it.op.mode, [&](auto m) {
-    b_smooth_colour64<m()>(it.n, it.phi, it.src, it.f, it.sc, it.op, colour, blk);
+    cell_smooth64<m()>(it.n, it.phi, it.src, it.f, s_c, it.op, colour, blk * 256 + threadIdx.x);
   });
 }
 
-__global__ void __launch_bounds__(256) kb_residual_restrict64(const BItem* __restrict__ items,
-                                                              int count) {
+__global__ void __launch_bounds__(256, 4) kb_smooth_tile64(const BItem* __restrict__ items,
+                                                           int count, int colour) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
   __shared__ TileShared S;
-  if (in_tiles(it.n, it.op)) {
-    const int3 o = tile_origin(it.n, blk);
-    Partial p;
-    auto run = [&](auto f, auto lin) {
-      p = b_residual_restrict_tile64<decltype(f)::value, decltype(lin)::value>(
-          it.n, it.phi, it.src, it.f, it.op, it.cphi, it.cphihat, it.cf, o.x, o.y, o.z, S);
-    };
-    pick(it.f != nullptr, it.op.mode == OP_LINEAR, run);
-    if (threadIdx.x == 0) it.part[blk] = p;
-    return;
-  }
+  const int3 o = tile_origin(it.n, blk);
+  pick(it.f != nullptr, it.op.mode == OP_LINEAR, [&](auto f, auto lin) {
+    b_smooth_tile64<decltype(f)::value, decltype(lin)::value>(
+        it.n, it.phi, it.src, it.f, it.sc, it.op, colour, o.x, o.y, o.z, S);
+  });
+}
+
+__global__ void __launch_bounds__(256, 2) kb_residual_restrict64(const BItem* __restrict__ items,
+                                                                 int count) {
+  long long blk;
+  const BItem& it = find_item(items, count, blk);
   by_mode(it.op.mode, [&](auto m) {
     b_residual_restrict64<m()>(it.n, it.phi, it.src, it.f, it.op, it.cphi, it.cphihat, it.cf,
                                it.part, blk);
   });
+}
+
+__global__ void __launch_bounds__(256, 2) kb_residual_restrict_tile64(
+    const BItem* __restrict__ items, int count) {
+  long long blk;
+  const BItem& it = find_item(items, count, blk);
+  __shared__ TileShared S;
+  const int3 o = tile_origin(it.n, blk);
+  Partial p;
+  pick(it.f != nullptr, it.op.mode == OP_LINEAR, [&](auto f, auto lin) {
+    p = b_residual_restrict_tile64<decltype(f)::value, decltype(lin)::value>(
+        it.n, it.phi, it.src, it.f, it.op, it.cphi, it.cphihat, it.cf, o.x, o.y, o.z, S);
+  });
+  if (threadIdx.x == 0) it.part[blk] = p;
 }
 
 // One block per item.  mode 0: partials of a residual-restriction (one per 256
@@ -155,34 +166,41 @@ __global__ void __launch_bounds__(1024) kb_finalize(const BItem* __restrict__ it
   }
 }
 
-__global__ void __launch_bounds__(256) kb_fas_rhs64(const BItem* __restrict__ items, int count) {
+__global__ void __launch_bounds__(256, 3) kb_fas_rhs64(const BItem* __restrict__ items,
+                                                       int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
-  __shared__ TileShared S;
-  if (in_tiles(it.n / 2, it.cop)) {
-    const int3 o = tile_origin(it.n / 2, blk);
-    if (it.cop.mode == OP_LINEAR)
-      b_fas_rhs_tile64<true>(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, o.x, o.y,
-                             o.z, S);
-    else
-      b_fas_rhs_tile64<false>(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, o.x, o.y,
-                              o.z, S);
-    return;
-  }
   by_mode(it.cop.mode, [&](auto m) {
     b_fas_rhs64<m()>(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, blk);
   });
 }
 
+__global__ void __launch_bounds__(256, 4) kb_fas_rhs_tile64(const BItem* __restrict__ items,
+                                                            int count) {
+  long long blk;
+  const BItem& it = find_item(items, count, blk);
+  __shared__ TileShared S;
+  const int3 o = tile_origin(it.n / 2, blk);
+  if (it.cop.mode == OP_LINEAR)
+    b_fas_rhs_tile64<true>(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, o.x, o.y, o.z,
+                           S);
+  else
+    b_fas_rhs_tile64<false>(it.n / 2, it.cphi, it.csrc, it.cf, it.cop, it.sc, it.csc, o.x, o.y,
+                            o.z, S);
+}
+
 __global__ void __launch_bounds__(256) kb_prolong64(const BItem* __restrict__ items, int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
-  if (prolong_columns(it.n / 2)) {
-    const int3 o = column_block(it.n / 2, blk);
-    prolong_column<double, double2, 4>(it.n / 2, it.cphi, it.cphihat, it.phi, o.x, o.y, o.z);
-    return;
-  }
   b_prolong_correct64(it.n / 2, it.cphi, it.cphihat, it.phi, blk);
+}
+
+__global__ void __launch_bounds__(256) kb_prolong_column64(const BItem* __restrict__ items,
+                                                           int count) {
+  long long blk;
+  const BItem& it = find_item(items, count, blk);
+  const int3 o = column_block(it.n / 2, blk);
+  prolong_column<double, double2, 4>(it.n / 2, it.cphi, it.cphihat, it.phi, o.x, o.y, o.z);
 }
 
 __global__ void __launch_bounds__(256) kb_coarsest64(const BItem* __restrict__ items, int sweeps,
@@ -192,23 +210,28 @@ __global__ void __launch_bounds__(256) kb_coarsest64(const BItem* __restrict__ i
 }
 
 // ---- mixed-precision stages ----
-__global__ void __launch_bounds__(256) kb_handoff64(const BItem* __restrict__ items, int count) {
+__global__ void __launch_bounds__(256, 2) kb_handoff64(const BItem* __restrict__ items,
+                                                       int count) {
+  long long blk;
+  const BItem& it = find_item(items, count, blk);
+  const Handoff out{it.rhs, it.q0, it.phi0, it.e, nullptr, nullptr};
+  by_mode(it.op.mode, [&](auto m) {
+    b_residual_handoff64<m()>(it.n, it.phi, it.src, it.op, it.sc, out, it.part, blk);
+  });
+}
+
+__global__ void __launch_bounds__(256, 4) kb_handoff_tile64(const BItem* __restrict__ items,
+                                                            int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
   __shared__ TileShared S;
   const Handoff out{it.rhs, it.q0, it.phi0, it.e, nullptr, nullptr};
-  if (in_tiles(it.n, it.op)) {
-    const int3 o = tile_origin(it.n, blk);
-    const Partial p =
-        it.op.mode == OP_LINEAR
-            ? b_handoff_tile64<true>(it.n, it.phi, it.src, it.op, it.sc, out, o.x, o.y, o.z, S)
-            : b_handoff_tile64<false>(it.n, it.phi, it.src, it.op, it.sc, out, o.x, o.y, o.z, S);
-    if (threadIdx.x == 0) it.part[blk] = p;
-    return;
-  }
-  by_mode(it.op.mode, [&](auto m) {
-    b_residual_handoff64<m()>(it.n, it.phi, it.src, it.op, it.sc, out, it.part, blk);
-  });
+  const int3 o = tile_origin(it.n, blk);
+  const Partial p =
+      it.op.mode == OP_LINEAR
+          ? b_handoff_tile64<true>(it.n, it.phi, it.src, it.op, it.sc, out, o.x, o.y, o.z, S)
+          : b_handoff_tile64<false>(it.n, it.phi, it.src, it.op, it.sc, out, o.x, o.y, o.z, S);
+  if (threadIdx.x == 0) it.part[blk] = p;
 }
 
 __global__ void __launch_bounds__(256) kb_update64(const BItem* __restrict__ items, int count) {
@@ -255,8 +278,10 @@ __global__ void __launch_bounds__(256) kb_smooth32(const BItem* __restrict__ ite
                                bz);
 }
 
-__global__ void __launch_bounds__(256) kb_residual_restrict32(const BItem* __restrict__ items,
-                                                              int count) {
+// Three CTAs per SM: without the bound it takes 110 registers and two (mixed batches of 64
+// with boxes to 128^3 118.7 -> 116.2 ms, to 96^3 68.6 -> 67.7; of 32^3 alone 14.9 -> 15.1).
+__global__ void __launch_bounds__(256, 3) kb_residual_restrict32(const BItem* __restrict__ items,
+                                                                 int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
   b_residual_restrict32(it.n, it.e, it.phi0, it.q0, it.rhs, it.op32, it.ce, it.cehat, it.crhs,
@@ -272,12 +297,15 @@ __global__ void __launch_bounds__(256) kb_fas_rhs32(const BItem* __restrict__ it
 __global__ void __launch_bounds__(256) kb_prolong32(const BItem* __restrict__ items, int count) {
   long long blk;
   const BItem& it = find_item(items, count, blk);
-  if (prolong_columns(it.n / 2)) {
-    const int3 o = column_block(it.n / 2, blk);
-    prolong_column<float, float2, 4>(it.n / 2, it.ce, it.cehat, it.e, o.x, o.y, o.z);
-    return;
-  }
   b_prolong_correct32(it.n / 2, it.ce, it.cehat, it.e, blk);
+}
+
+__global__ void __launch_bounds__(256) kb_prolong_column32(const BItem* __restrict__ items,
+                                                           int count) {
+  long long blk;
+  const BItem& it = find_item(items, count, blk);
+  const int3 o = column_block(it.n / 2, blk);
+  prolong_column<float, float2, 4>(it.n / 2, it.ce, it.cehat, it.e, o.x, o.y, o.z);
 }
 
 __global__ void __launch_bounds__(256) kb_coarsest_corr32(const BItem* __restrict__ items,
@@ -289,44 +317,62 @@ __global__ void __launch_bounds__(256) kb_coarsest_corr32(const BItem* __restric
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-// T_HAND: the outer residual hand-off, kHandoffCells cells per thread
-// T_PROLONG: the prolongations, by columns where they run so;
-// T_SM64, T_RR64, T_CCELL64: the FP64 colour stages, residual restrictions and right-hand
-// sides (of the level below), and T_HAND: in tiles from kTileMinSide on
+// The work lists: each stage's items, those in tiles (T_*_TILE, from kTileMinSide on) or by
+// columns (T_PROLONG_COL) apart.  T_SM64, T_RR64, T_CCELL64: the FP64 colour stages, residual
+// restrictions and right-hand sides (of the level below); T_HAND: the outer residual's
+// hand-off, kHandoffCells cells per thread.
 enum ListType {
-  T_SMOOTH = 0, T_RR, T_CELL, T_CCELL, T_ONE, T_HAND, T_SM64, T_RR64, T_CCELL64,
-  T_PROLONG, T_NTYPES
+  T_SMOOTH = 0, T_RR, T_CELL, T_CCELL, T_ONE, T_HAND, T_HAND_TILE, T_SM64, T_SM64_TILE,
+  T_RR64, T_RR64_TILE, T_CCELL64, T_CCELL64_TILE, T_PROLONG, T_PROLONG_COL, T_NTYPES
 };
 
+// Whether solves of this precision launch a list of level l.
+static bool list_used(ListType t, int l, bool mixed) {
+  switch (t) {
+    case T_ONE:
+    case T_PROLONG:
+    case T_PROLONG_COL: return true;
+    case T_HAND:
+    case T_HAND_TILE: return mixed && l == 0;
+    case T_SMOOTH:
+    case T_RR:
+    case T_CELL:
+    case T_CCELL: return mixed;
+    default: return !mixed;
+  }
+}
+
+// The blocks of an item in a list, 0 where it belongs to the stage's other one.
 static long long blocks_of(ListType t, const BItem& it) {
   const int n = it.n;
   const long long cells = (long long)n * n * n;
+  auto tiled = [](bool tiles, int side) { return tiles ? (long long)tile_count(side) : 0; };
+  auto plain = [](bool tiles, long long work) { return tiles ? 0 : (work + 255) / 256; };
+  const bool t_s = smooth_in_tiles(n, it.op), t_r = in_tiles(n, it.op);
+  const bool t_c = in_tiles(n / 2, it.cop), cols = prolong_columns(n / 2);
   switch (t) {
-    case T_SM64:
-      if (smooth_in_tiles(n, it.op)) return tile_count(n);
-      return (cells / 4 + 255) / 256;
+    case T_SM64: return plain(t_s, cells / 4);
+    case T_SM64_TILE: return tiled(t_s, n);
+    case T_RR64: return plain(t_r, cells / 8);
+    case T_RR64_TILE: return tiled(t_r, n);
+    case T_CCELL64: return plain(t_c, cells / 8);
+    case T_CCELL64_TILE: return tiled(t_c, n / 2);
+    case T_HAND: return plain(t_r, (cells + kHandoffCells - 1) / kHandoffCells);
+    case T_HAND_TILE: return tiled(t_r, n);
     case T_SMOOTH: {
       if (n < kColour32TileMin) return (cells / 4 + 255) / 256;
       const dim3 g = colour32_narrow(n) ? colour32_grid<16>(n) : colour32_grid<32>(n);
       return (long long)g.x * g.y * g.z;
     }
-    case T_RR64:
-      if (in_tiles(n, it.op)) return tile_count(n);
-      return (cells / 8 + 255) / 256;
-    case T_RR: return (cells / 8 + 255) / 256;
+    case T_RR:
+    case T_CCELL: return (cells / 8 + 255) / 256;
     case T_CELL: return (cells + 255) / 256;
-    case T_PROLONG: {
-      if (!prolong_columns(n / 2)) return (cells + 255) / 256;
+    case T_PROLONG: return plain(cols, cells);
+    case T_PROLONG_COL: {
+      if (!cols) return 0;
       const dim3 g = prolong_grid(n / 2, 4);
       return (long long)g.x * g.y * g.z;
     }
-    case T_CCELL64:
-      if (in_tiles(n / 2, it.cop)) return tile_count(n / 2);
-      return (cells / 8 + 255) / 256;
-    case T_CCELL: return (cells / 8 + 255) / 256;
-    case T_HAND:
-      if (in_tiles(n, it.op)) return tile_count(n);
-      return (cells + 256 * kHandoffCells - 1) / (256 * kHandoffCells);
     default: return 1;
   }
 }
@@ -339,8 +385,11 @@ struct StageList {
 };
 
 struct BatchState {
-  std::vector<StageList> lists;  // [level][type][pred]
+  std::vector<StageList> lists;  // [level][type], in d_items
   StageList coarsest;
+  BItem* d_items = nullptr;  // of all lists, and what it is copied from
+  std::vector<BItem> items;
+  size_t capacity = 0;
   int lmax = 0;
   LevelScalars* d_out = nullptr;
   LevelScalars* h_out = nullptr;
@@ -349,19 +398,11 @@ struct BatchState {
   long long na = 0, nb = 0;
 };
 
-// which solves an item list holds: the level exists (P_HAS) or is above the
-// solve's coarsest (P_DESC)
-enum Pred { P_HAS = 0, P_DESC = 1 };
-
-static StageList& list_at(BatchState* bs, int l, ListType t, Pred p) {
-  return bs->lists[((size_t)l * T_NTYPES + t) * 2 + p];
+static StageList& list_at(BatchState* bs, int l, ListType t) {
+  return bs->lists[(size_t)l * T_NTYPES + t];
 }
 
-static void free_lists(BatchState* bs) {
-  for (auto& L : bs->lists) cudaFree(L.d);
-  bs->lists.clear();
-  cudaFree(bs->coarsest.d);
-  bs->coarsest = StageList();
+static void free_graphs(BatchState* bs) {
   if (bs->ga) cudaGraphExecDestroy(bs->ga);
   if (bs->gb) cudaGraphExecDestroy(bs->gb);
   bs->ga = bs->gb = nullptr;
@@ -387,7 +428,8 @@ mg_status batch_prepare(mg_grid* g) {
 void batch_release(mg_grid* g) {
   BatchState* bs = g->bs;
   if (!bs) return;
-  free_lists(bs);
+  free_graphs(bs);
+  cudaFree(bs->d_items);
   cudaFree(bs->d_out);
   if (bs->h_out) cudaFreeHost(bs->h_out);
   delete bs;
@@ -444,61 +486,66 @@ static BItem make_item(mg_grid* g, const SolveParams& P, int s, int l) {
   return it;
 }
 
-static mg_status upload(StageList& L, std::vector<BItem>& items) {
-  cudaFree(L.d);
-  L.d = nullptr;
-  L.count = (int)items.size();
-  if (items.empty()) return MG_OK;
-  if (cudaMalloc(&L.d, sizeof(BItem) * items.size()) != cudaSuccess) {
-    set_error("batch: work-list allocation");
-    return MG_ENOMEM;
+// The work lists of the active solves, in one buffer and one copy on the handle's stream (no
+// work of the batch is under way there).  A level's lists hold the solves that go below it,
+// T_HAND's and T_CELL's those that have it.
+static mg_status build_lists(mg_grid* g, const SolveParams& P) {
+  BatchState* bs = g->bs;
+  free_graphs(bs);
+  bs->lists.assign((size_t)bs->lmax * T_NTYPES, StageList());
+  const bool mixed = !P.ops32.empty();
+  std::vector<BItem>& items = bs->items;
+  items.clear();
+  std::vector<size_t> first;
+  for (int l = 0; l < bs->lmax; ++l) {
+    std::vector<BItem> level;  // of the solves that have it
+    std::vector<char> below;
+    for (int s : bs->active)
+      if (l < g->domains[s]->nlev) {
+        level.push_back(make_item(g, P, s, l));
+        below.push_back(l < g->domains[s]->nlev - 1);
+      }
+    for (int t = 0; t < T_NTYPES; ++t) {
+      StageList& L = list_at(bs, l, (ListType)t);
+      first.push_back(items.size());
+      if (!list_used((ListType)t, l, mixed)) continue;
+      const bool has = t == T_CELL || t == T_HAND || t == T_HAND_TILE;
+      for (size_t k = 0; k < level.size(); ++k) {
+        const long long blocks = has || below[k] ? blocks_of((ListType)t, level[k]) : 0;
+        if (blocks == 0) continue;
+        items.push_back(level[k]);
+        items.back().block0 = (int)L.blocks;
+        L.blocks += blocks;
+        L.count += 1;
+      }
+    }
   }
-  if (cudaMemcpy(L.d, items.data(), sizeof(BItem) * items.size(), cudaMemcpyHostToDevice) !=
-      cudaSuccess) {
+  first.push_back(items.size());
+  bs->coarsest = StageList();
+  for (int s : bs->active) {
+    items.push_back(make_item(g, P, s, g->domains[s]->nlev - 1));
+    items.back().block0 = bs->coarsest.count++;
+    bs->coarsest.maxn = std::max(bs->coarsest.maxn, items.back().n);
+  }
+  bs->coarsest.blocks = bs->coarsest.count;
+  if (items.size() > bs->capacity) {
+    cudaFree(bs->d_items);
+    bs->d_items = nullptr;
+    bs->capacity = 0;
+    if (cudaMalloc(&bs->d_items, sizeof(BItem) * items.size()) != cudaSuccess) {
+      set_error("batch: work-list allocation");
+      return MG_ENOMEM;
+    }
+    bs->capacity = items.size();
+  }
+  if (cudaMemcpyAsync(bs->d_items, items.data(), sizeof(BItem) * items.size(),
+                      cudaMemcpyHostToDevice, g->stream) != cudaSuccess) {
     set_error("batch: work-list upload");
     return MG_ECUDA;
   }
+  for (size_t k = 0; k < bs->lists.size(); ++k) bs->lists[k].d = bs->d_items + first[k];
+  bs->coarsest.d = bs->d_items + first.back();
   return MG_OK;
-}
-
-static mg_status build_lists(mg_grid* g, const SolveParams& P) {
-  BatchState* bs = g->bs;
-  free_lists(bs);
-  bs->lists.resize((size_t)bs->lmax * T_NTYPES * 2);
-  for (int l = 0; l < bs->lmax; ++l)
-    for (int t = 0; t < T_NTYPES; ++t)
-      for (int p = 0; p < 2; ++p) {
-        std::vector<BItem> items;
-        long long blocks = 0;
-        int maxn = 0;
-        for (int s : bs->active) {
-          const int nl = g->domains[s]->nlev;
-          const bool ok = (p == P_HAS) ? (l < nl) : (l < nl - 1);
-          if (!ok) continue;
-          BItem it = make_item(g, P, s, l);
-          it.block0 = (int)blocks;
-          blocks += blocks_of((ListType)t, it);
-          maxn = std::max(maxn, it.n);
-          items.push_back(it);
-        }
-        StageList& L = list_at(bs, l, (ListType)t, (Pred)p);
-        mg_status st = upload(L, items);
-        if (st != MG_OK) return st;
-        L.blocks = blocks;
-        L.maxn = maxn;
-      }
-  std::vector<BItem> co;
-  int maxn = 0;
-  for (int s : bs->active) {
-    BItem it = make_item(g, P, s, g->domains[s]->nlev - 1);
-    it.block0 = (int)co.size();
-    maxn = std::max(maxn, it.n);
-    co.push_back(it);
-  }
-  mg_status st = upload(bs->coarsest, co);
-  bs->coarsest.blocks = (long long)co.size();
-  bs->coarsest.maxn = maxn;
-  return st;
 }
 
 struct BatchCycle {
@@ -507,17 +554,18 @@ struct BatchCycle {
   const mg_options* o;
   cudaStream_t st;
 
-  const StageList& L(int l, ListType t, Pred p) const { return list_at(bs, l, t, p); }
+  const StageList& L(int l, ListType t) const { return list_at(bs, l, t); }
 
   template <typename K, typename... A>
-  void launch(const StageList& sl, int threads, K kernel, A... args) const {
+  void launch(int l, ListType t, K kernel, A... args) const {
+    const StageList& sl = L(l, t);
     if (sl.count == 0) return;
-    kernel<<<(unsigned)sl.blocks, threads, 0, st>>>(sl.d, sl.count, args...);
+    kernel<<<(unsigned)sl.blocks, 256, 0, st>>>(sl.d, sl.count, args...);
     count_launches(1);
   }
 
-  void finalize(int l, ListType src_type, int mode, int use32, int clear_mu) const {
-    const StageList& one = L(l, T_ONE, src_type == T_RR ? P_DESC : P_HAS);
+  void finalize(int l, int mode, int use32, int clear_mu) const {
+    const StageList& one = L(l, T_ONE);
     if (one.count == 0) return;
     kb_finalize<<<one.count, 1024, 0, st>>>(one.d, mode, use32, clear_mu);
     count_launches(1);
@@ -526,22 +574,32 @@ struct BatchCycle {
   // ---- FP64 ----
   void smooth64(int l, int sweeps) const {
     for (int s = 0; s < sweeps; ++s)
-      for (int c = 0; c < 4; ++c) launch(L(l, T_SM64, P_DESC), 256, kb_smooth64, c);
+      for (int c = 0; c < 4; ++c) {
+        launch(l, T_SM64_TILE, kb_smooth_tile64, c);
+        launch(l, T_SM64, kb_smooth64, c);
+      }
+  }
+  void residual64(int l) const {
+    launch(l, T_RR64_TILE, kb_residual_restrict_tile64);
+    launch(l, T_RR64, kb_residual_restrict64);
+    finalize(l, 0, 0, 0);
+  }
+  void rhs64(int l) const {
+    launch(l, T_CCELL64_TILE, kb_fas_rhs_tile64);
+    launch(l, T_CCELL64, kb_fas_rhs64);
   }
   void part_a64() const {
     smooth64(0, o->nu_pre);
-    launch(L(0, T_RR64, P_DESC), 256, kb_residual_restrict64);
-    finalize(0, T_RR, 0, 0, 0);
+    residual64(0);
     cudaMemcpyAsync(bs->h_out, bs->d_out, sizeof(LevelScalars) * g->domains.size(),
                     cudaMemcpyDeviceToHost, st);
   }
   void part_b64() const {
-    launch(L(0, T_CCELL64, P_DESC), 256, kb_fas_rhs64);
+    rhs64(0);
     for (int l = 1; l < bs->lmax - 1; ++l) {
       smooth64(l, o->nu_pre);
-      launch(L(l, T_RR64, P_DESC), 256, kb_residual_restrict64);
-      finalize(l, T_RR, 0, 0, 0);
-      launch(L(l, T_CCELL64, P_DESC), 256, kb_fas_rhs64);
+      residual64(l);
+      rhs64(l);
     }
     const size_t smem = 3 * sizeof(double) * (size_t)bs->coarsest.maxn * bs->coarsest.maxn *
                         bs->coarsest.maxn;
@@ -549,7 +607,8 @@ struct BatchCycle {
                                                          o->coarse_drop);
     count_launches(1);
     for (int l = bs->lmax - 2; l >= 0; --l) {
-      launch(L(l, T_PROLONG, P_DESC), 256, kb_prolong64);
+      launch(l, T_PROLONG_COL, kb_prolong_column64);
+      launch(l, T_PROLONG, kb_prolong64);
       smooth64(l, o->nu_post);
     }
   }
@@ -557,20 +616,21 @@ struct BatchCycle {
   // ---- mixed ----
   void smooth32(int l, int sweeps) const {
     for (int s = 0; s < sweeps; ++s)
-      for (int c = 0; c < 4; ++c) launch(L(l, T_SMOOTH, P_DESC), 256, kb_smooth32, c);
+      for (int c = 0; c < 4; ++c) launch(l, T_SMOOTH, kb_smooth32, c);
   }
   void part_a_mixed() const {
-    launch(L(0, T_HAND, P_HAS), 256, kb_handoff64);
-    finalize(0, T_HAND, 2, 0, 1);
+    launch(0, T_HAND_TILE, kb_handoff_tile64);
+    launch(0, T_HAND, kb_handoff64);
+    finalize(0, 2, 0, 1);
     cudaMemcpyAsync(bs->h_out, bs->d_out, sizeof(LevelScalars) * g->domains.size(),
                     cudaMemcpyDeviceToHost, st);
   }
   void inner() const {
     for (int l = 0; l < bs->lmax - 1; ++l) {
       smooth32(l, o->nu_pre);
-      launch(L(l, T_RR, P_DESC), 256, kb_residual_restrict32);
-      finalize(l, T_RR, 0, 1, 0);
-      launch(L(l, T_CCELL, P_DESC), 256, kb_fas_rhs32);
+      launch(l, T_RR, kb_residual_restrict32);
+      finalize(l, 0, 1, 0);
+      launch(l, T_CCELL, kb_fas_rhs32);
     }
     const size_t smem = 4 * sizeof(double) * (size_t)bs->coarsest.maxn * bs->coarsest.maxn *
                         bs->coarsest.maxn;
@@ -578,17 +638,18 @@ struct BatchCycle {
                                                               o->coarse_drop);
     count_launches(1);
     for (int l = bs->lmax - 2; l >= 0; --l) {
-      launch(L(l, T_PROLONG, P_DESC), 256, kb_prolong32);
+      launch(l, T_PROLONG_COL, kb_prolong_column32);
+      launch(l, T_PROLONG, kb_prolong32);
       smooth32(l, o->nu_post);
     }
   }
   void part_b_mixed() const {
     for (int l = 1; l < bs->lmax; ++l) {
-      launch(L(l - 1, T_CCELL, P_DESC), 256, kb_restrict_phi0);
-      launch(L(l, T_CELL, P_HAS), 256, kb_q0_prep);
+      launch(l - 1, T_CCELL, kb_restrict_phi0);
+      launch(l, T_CELL, kb_q0_prep);
     }
     for (int c = 0; c < o->inner_cycles; ++c) inner();
-    launch(L(0, T_CELL, P_HAS), 256, kb_update64);
+    launch(0, T_CELL, kb_update64);
   }
 };
 

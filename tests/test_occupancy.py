@@ -57,3 +57,13 @@ def ctas(tmp_path_factory):
     ("k_smooth_colour64", SQRT, 3), ("k_residual_restrict64", SQRT, 2)])
 def test_one_form_does_not_carry_the_others(ctas, kernel, mode, least):
     assert ctas("mg_fp64.cu", kernel, mode) >= least
+
+
+@pytest.mark.parametrize("kernel,least", [
+    ("kb_smooth64", 3), ("kb_smooth_tile64", 4), ("kb_residual_restrict64", 2),
+    ("kb_residual_restrict_tile64", 2), ("kb_fas_rhs64", 3), ("kb_fas_rhs_tile64", 4),
+    ("kb_handoff64", 2), ("kb_handoff_tile64", 4), ("kb_prolong64", 6), ("kb_prolong_column64", 3),
+    ("kb_prolong32", 8), ("kb_prolong_column32", 5), ("kb_residual_restrict32", 3),
+    ("kb_smooth32", 5)])
+def test_batch_stages_in_tiles_and_cell_by_cell(ctas, kernel, least):
+    assert ctas("mg_batch.cu", kernel) >= least
