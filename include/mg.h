@@ -60,7 +60,12 @@ typedef enum {
 
 typedef enum {
   MG_FP64 = 0,  /* every step in FP64 */
-  MG_MIXED = 1  /* FP32 correction V-cycles inside an FP64 defect-correction loop */
+  MG_MIXED = 1  /* FP32 correction V-cycles inside an FP64 defect-correction loop.  The first
+                   such solve of a handle takes 4 to 5 FP32 arrays of every level and, for
+                   sides from 64 on, two more of the finest (8 bytes per cell; not in a
+                   batch).  The solve does without those two, a little slower, where they
+                   cannot be had and, for sides that are no power of two, where more than half
+                   of the device's memory is taken already. */
 } mg_precision;
 
 /*
