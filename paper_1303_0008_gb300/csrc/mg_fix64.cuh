@@ -326,10 +326,12 @@ MG_HD long long tile_convert(long long b, int em) {
 
 // The high word of a tile value's magnitude, and the bounds that one of the six across a cell's
 // faces has to reach, or the unit would be too coarse for the cell: 2^-7 of the tile's range
-// for an update, where six rounded values count a sixth each, and 2^-6 for a defect (there
-// the centre's may do as well), to which the centre adds six times its own rounding.
+// for an update, where six rounded values count a sixth each, and 2^-6 for a defect, to which
+// the centre adds six times its own rounding.  A defect's centre of 2^-8 of the range will do
+// too: it is exact, and six times it is the largest term.
 MG_HD unsigned tile_mag(long long v) { return (unsigned)(fix_hi(v) ^ (fix_hi(v) >> 31)); }
-constexpr unsigned kTileSmall = 1u << 21, kTileSmallDefect = 1u << 22;
+constexpr unsigned kTileSmall = 1u << 21, kTileSmallDefect = 1u << 22,
+                   kTileSmallCentre = 1u << 20;
 
 #ifdef __CUDACC__
 static __device__ __noinline__ float fix_to_float_rare(double x) { return (float)x; }

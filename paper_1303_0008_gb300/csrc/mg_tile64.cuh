@@ -11,13 +11,13 @@
 //
 // Values within 2^-7 of the tile's largest keep all their bits; the others are rounded to the
 // unit.  That loses less than FP64 additions do as long as one of the six neighbours
-// across a face reaches 2^-7 of the tile's largest (2^-6 for a defect); tile_small finds the
-// other cells (those at a zero of the field in a steep tile), which take their values from
-// memory.  In units of
-// 2^-53 of an update's largest term, the error of a cell (rms and worst of 160000) where
-// 1.07 and 5.3 are FP64's: 0.88 and 4.2 on noise whose amplitude falls as exp(-0.15 i - 0.1 j)
-// through the tile (with the values cut off instead of rounded 1.14 and 6.5), 0.89 and 3.8 on
-// noise of one amplitude.
+// across a face reaches 2^-7 of the tile's largest (for a defect 2^-6, or its centre 2^-8);
+// tile_small finds the other cells (those at a zero of the field in a steep tile), which take
+// their values from memory.  In units of 2^-53 of an update's largest term, the error of a cell
+// (rms and worst of 160000) where 1.07 and 5.3 are FP64's: 0.88 and 4.2 on noise whose amplitude
+// falls as exp(-0.15 i - 0.1 j) through the tile (with the values cut off instead of rounded
+// 1.14 and 6.5), 0.89 and 3.8 on noise of one amplitude.  The rounding costs a colour stage
+// 0.8 % (256^3 76.9 -> 77.6 us).
 // Tiles without such a unit (infinities, NaN, extreme exponents) go cell by cell too.
 #pragma once
 
@@ -303,9 +303,10 @@ __device__ __forceinline__ void b_smooth_tile64(int n, double* __restrict__ phi,
     }
   }
 #pragma unroll 1
-  for (int s = 0; rare != 0; ++s, rare >>= 1) {
-    const int k = k0 + 2 * s;
-    if ((rare & 1) && k < n) cell_smooth64_at<LIN ? OP_LINEAR : OP_SQRT>(n, phi, src, f, s_c, c, i, j, k);
+  for (; rare != 0; rare &= rare - 1) {
+    const int k = k0 + 2 * (__ffs((int)rare) - 1);
+    if (k < n)
+      cell_smooth64_at<LIN ? OP_LINEAR : OP_SQRT>(n, phi, src, f, s_c, c, i, j, k);
   }
 }
 
@@ -405,7 +406,7 @@ __device__ __forceinline__ bool tile_defect(const long long* q, const TilePlane&
   const unsigned ls = (unsigned)(fix_hi(lap) >> 31);
   const u64 lm = ((u64)lap ^ fix_words(ls, ls)) - fix_words(ls, ls);
   bool bad = min((unsigned)(lm >> 32), tq) == 0 ||
-             ((tile_mag((long long)mid.c) << 3 | tq) < 8 * kTileSmallDefect &&
+             (tile_mag((long long)mid.c) < kTileSmallCentre && tq < 8 * kTileSmallDefect &&
               tile_small(q, 0, -1, 1, kTileSmallDefect));
   double D = src;
   qd = 1.0;
@@ -418,12 +419,16 @@ __device__ __forceinline__ bool tile_defect(const long long* q, const TilePlane&
   return !bad;
 }
 
-// The defect kernels, 512^3: residual 13.1 -> 1.65 ms, residual with restriction 10.5 ->
-// 2.32 ms, hand-off to FP32 10.5 -> 3.11 ms (256^3 residual 1646 -> 220 us).  Per cell three
+// The defect kernels, 512^3: residual 13.1 -> 1.69 ms, residual with restriction 10.5 ->
+// 2.21 ms, hand-off to FP32 10.5 -> 2.10 ms (256^3 residual 1646 -> 234 us).  Per cell three
 // to five FP64 instructions remain (the FP64 pipe is about half busy) beside some 430 others,
-// two thirds of the issue slots.  Four CTAs per SM at 64 registers against three at 80:
-// residual 1.65 against 1.80 ms, hand-off 3.11 against 3.28 ms; the restriction, which keeps
-// two columns at once, is fastest at two.
+// two thirds of the issue slots.  Four CTAs per SM at 64 registers against three at 80 (when
+// chosen): residual 1.65 against 1.80 ms, hand-off 3.11 against 3.28 ms; the restriction, which
+// keeps two columns at once, is fastest at two.
+//
+// Of the cells that need another path each lane takes the next of its own: a warp then
+// evaluates as many as its worst lane has, not one for every place where some lane has one
+// (512^3: restriction 2.70 -> 2.34 ms, 128^3: 60 -> 51 us; colour stages 571 -> 566 us).
 //
 // Visit every cell of the tile at (x0, y0, z0): cell(id, i, j, k, defect, q, guard) with
 // src(id) its source term.  A thread takes two columns of eight cells, side by side in y,
@@ -462,9 +467,10 @@ __device__ __forceinline__ void tile_defects(int n, const double* __restrict__ p
     }
   }
 #pragma unroll 1
-  for (int s = 0; rare != 0; ++s, rare >>= 1) {
+  for (; rare != 0; rare &= rare - 1) {
+    const int s = __ffs((int)rare) - 1;
     const int j = j0 + (s >> 3), k = z0 + (s & 7);
-    if (!(rare & 1) || k >= n) continue;
+    if (k >= n) continue;
     const int id = k * n2 + j * n + i;
     double qd, d;
     bool g;
@@ -532,28 +538,42 @@ __device__ __forceinline__ Partial b_residual_restrict_tile64(
     double sd = 0.0;
     unsigned long long sphi = 0;
     if (in) {
+      auto place = [&](int ch) { return (k0 + (ch >> 1)) * n2 + (j0 + (ch & 1)) * nf + i; };
+      double dv[4];
+      unsigned rare = 0xf;
+      if (ok) {
+        rare = 0;
 #pragma unroll
-      for (int ch = 0; ch < 4; ++ch) {
-        const int y = ch & 1, k = k0 + (ch >> 1), j = j0 + y;
-        const int id = k * n2 + j * nf + i;
-        double qd, d;
-        bool g = false, good = false;
-        if (ok) {
+        for (int ch = 0; ch < 4; ++ch) {
+          const int y = ch & 1;
+          double qd;
           const TilePlane up = tile_plane(q[y] + kTilePlane);
-          good = tile_defect<LIN>(q[y], lo[y], mid[y], up, ue, src[id], c, d, qd);
+          if (!tile_defect<LIN>(q[y], lo[y], mid[y], up, ue, src[place(ch)], c, dv[ch], qd))
+            rare |= 1u << ch;
           sphi += mid[y].c;
           lo[y] = mid[y];
           mid[y] = up;
           q[y] += kTilePlane;
         }
-        if (!good) d = tile_defect_rare<LIN>(phi, nf, i, j, k, src[id], &c, &g);
-        if (F) d -= f[id];
+      }
+#pragma unroll 1
+      for (; rare != 0; rare &= rare - 1) {  // as in tile_defects
+        const int r = __ffs((int)rare) - 1;
+        bool g;
+        const double d = tile_defect_rare<LIN>(phi, nf, i, j0 + (r & 1), k0 + (r >> 1),
+                                               src[place(r)], &c, &g);
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) dv[ch] = ch == r ? d : dv[ch];
+        p.guards += g ? 1 : 0;
+      }
+#pragma unroll
+      for (int ch = 0; ch < 4; ++ch) {
+        const double d = F ? dv[ch] - f[place(ch)] : dv[ch];
         const bool fin = finite_bits(d);
         const long long key = order_key(d);
         kmax = (fin && key > kmax) ? key : kmax;
         kmin = (fin && key < kmin) ? key : kmin;
         p.nonfinite += fin ? 0 : 1;
-        p.guards += g ? 1 : 0;
         sd += d;
       }
     }

@@ -34,8 +34,8 @@ static bool forms(const ll* v, unsigned small, bool defect, ll& face, u64& N, in
   unsigned tq, mag = 0;
   N = fix_quad(a, c, sh, tq);
   for (int k = 0; k < 6; ++k) mag |= tile_mag(v[k]);
-  const unsigned big = defect ? tile_mag(v[18]) << 3 : tile_mag(face);
-  return tq != 0 && face != 0 && !((big | tq) < (small << 3) && mag < small);
+  const bool low = defect ? tile_mag(v[18]) < kTileSmallCentre : tile_mag(face) < (small << 3);
+  return tq != 0 && face != 0 && !(low && tq < (small << 3) && mag < small);
 }
 
 // p: a tile and its shell, X x Y x Z; src: the source term.  Per inner cell the error of the
