@@ -296,8 +296,8 @@ __device__ __forceinline__ float gal_offdiag(const float* __restrict__ J, const 
   const int t = i + B * (j + B * k);
   // The patches that hold the 26 neighbours, then their values and the row, then the sum:
   // each group of loads is under way at once.  (With the test for a missing patch between
-  // each pair of dependent loads, a colour of 16384 patches took 9.7 us at B = 2 and 19.0 us
-  // at B = 4; now 5.8 and 13.4 us.)
+  // each pair of dependent loads, a colour of 16384 patches took 11.4 us at B = 2 and 26.3 us
+  // at B = 4; now 7.2 and 20.5 us.)
   int at[27];
 #pragma unroll
   for (int o = 0; o < 27; ++o) {
