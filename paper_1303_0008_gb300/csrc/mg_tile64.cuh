@@ -26,9 +26,11 @@
 namespace mg {
 
 // Levels from this side on run in tiles (a rule on the side alone, so that every caller
-// gives a level the same bits).  Smaller ones have too few tiles to fill the GPU twice:
-// at 96 a colour stage takes 14.0 us in 216 tiles and 12.9 us cell by cell, at 112 14.4
-// against 16.8 us, at 128 15.8 against 19.6 us.
+// gives a level the same bits).  Smaller ones have too few tiles to fill the GPU: at 112, 392
+// tiles, a colour stage takes 13.9 us in tiles and 16.7 us cell by cell (residual 43.5 against
+// 70.0), at 128 14.3 against 22.7 us.  The line was drawn where 96 took 14.0 against 12.9 us;
+// with one kernel per form and the rare cells lane by lane it takes 9.9 against 12.9 (residual
+// 27.5 against 44.5), so it could lie lower.
 constexpr int kTileMinSide = 112;
 
 constexpr int kTileX = 32, kTileY = 16, kTileZ = 8;
